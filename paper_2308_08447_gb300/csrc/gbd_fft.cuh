@@ -53,16 +53,79 @@
 
 namespace gbd {
 
-__device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
+// Arithmetic on two FP32 values in one instruction (PTX f32x2, sm_100 and later): the same FMA-pipe
+// time as two scalar instructions, but one issue slot.
+__device__ __forceinline__ unsigned long long f2_bits(float2 a) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a.x), "f"(a.y));
+  return r;
+}
+__device__ __forceinline__ float2 f2_of(unsigned long long u) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(u));
+  return r;
+}
+__device__ __forceinline__ float2 padd(float2 a, float2 b) {
+  unsigned long long r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(f2_bits(a)), "l"(f2_bits(b)));
+  return f2_of(r);
+}
+__device__ __forceinline__ float2 psub(float2 a, float2 b) {
+  unsigned long long r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(f2_bits(a)), "l"(f2_bits(b)));
+  return f2_of(r);
+}
+__device__ __forceinline__ float2 pmul(float2 a, float2 b) {
+  unsigned long long r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(f2_bits(a)), "l"(f2_bits(b)));
+  return f2_of(r);
+}
+__device__ __forceinline__ float2 pfma(float2 a, float2 b, float2 c) {
+  unsigned long long r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(f2_bits(a)), "l"(f2_bits(b)), "l"(f2_bits(c)));
+  return f2_of(r);
+}
+__device__ __forceinline__ float2 pdup(float v) { return make_float2(v, v); }
+__device__ __forceinline__ float2 pneg(float2 a) { return make_float2(-a.x, -a.y); }
+
+// A complex value is a float2 (re, im), or, where a thread transforms two lines at once, a cpair:
+// the real parts of the two lines and their imaginary parts, so that every operation is packed.
+struct __align__(16) cpair {
+  float2 x, y;
+};
+__device__ __forceinline__ float2 cadd(float2 a, float2 b) { return padd(a, b); }
+__device__ __forceinline__ float2 csub(float2 a, float2 b) { return psub(a, b); }
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
   return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
 }
 __device__ __forceinline__ float2 cconj(float2 a) { return make_float2(a.x, -a.y); }
 __device__ __forceinline__ float2 cscale(float2 a, float s) { return make_float2(a.x * s, a.y * s); }
+__device__ __forceinline__ float2 cfma(float s, float2 a, float2 b) {   // s a + b
+  return make_float2(fmaf(s, a.x, b.x), fmaf(s, a.y, b.y));
+}
 template <int S>
 __device__ __forceinline__ float2 cmul_i(float2 a) {  // a * (S i)
   return S > 0 ? make_float2(-a.y, a.x) : make_float2(a.y, -a.x);
+}
+template <int S>
+__device__ __forceinline__ float2 cadd_i(float2 a, float2 b) {  // a + S i b
+  return S > 0 ? make_float2(a.x - b.y, a.y + b.x) : make_float2(a.x + b.y, a.y - b.x);
+}
+__device__ __forceinline__ cpair cadd(cpair a, cpair b) { return {padd(a.x, b.x), padd(a.y, b.y)}; }
+__device__ __forceinline__ cpair csub(cpair a, cpair b) { return {psub(a.x, b.x), psub(a.y, b.y)}; }
+__device__ __forceinline__ cpair cmul(cpair a, float2 w) {
+  const float2 wx = pdup(w.x), wy = pdup(w.y);
+  return {pfma(a.x, wx, pneg(pmul(a.y, wy))), pfma(a.x, wy, pmul(a.y, wx))};
+}
+__device__ __forceinline__ cpair cscale(cpair a, float s) { return {pmul(a.x, pdup(s)), pmul(a.y, pdup(s))}; }
+__device__ __forceinline__ cpair cfma(float s, cpair a, cpair b) { return {pfma(pdup(s), a.x, b.x), pfma(pdup(s), a.y, b.y)}; }
+template <int S>
+__device__ __forceinline__ cpair cmul_i(cpair a) {
+  return S > 0 ? cpair{pneg(a.y), a.x} : cpair{a.y, pneg(a.x)};
+}
+template <int S>
+__device__ __forceinline__ cpair cadd_i(cpair a, cpair b) {
+  return S > 0 ? cpair{psub(a.x, b.y), padd(a.y, b.x)} : cpair{padd(a.x, b.y), psub(a.y, b.x)};
 }
 
 // L over its largest power-of-two factor (no recursion, so that it folds wherever L is known)
@@ -124,46 +187,46 @@ __host__ __device__ constexpr int line_stride() {
   return (L + L / 16) + (LF ? ((L + L / 16) % 2 == 0 ? 1 : 0) : 0);
 }
 
-// ---- register DFTs of size 2, 4, 8, 16 (sign S) -----------------------------------------
-template <int S>
-__device__ __forceinline__ void dft4(float2* x) {
-  float2 a0 = cadd(x[0], x[2]), a1 = csub(x[0], x[2]);
-  float2 b0 = cadd(x[1], x[3]), b1 = cmul_i<S>(csub(x[1], x[3]));
+// ---- register DFTs (sign S); V is float2 or cpair ---------------------
+template <int S, class V>
+__device__ __forceinline__ void dft4(V* x) {
+  const V a0 = cadd(x[0], x[2]), a1 = csub(x[0], x[2]);
+  const V b0 = cadd(x[1], x[3]), b1 = csub(x[1], x[3]);
   x[0] = cadd(a0, b0);
   x[2] = csub(a0, b0);
-  x[1] = cadd(a1, b1);
-  x[3] = csub(a1, b1);
+  x[1] = cadd_i<S>(a1, b1);
+  x[3] = cadd_i<-S>(a1, b1);
 }
 
-// X[q] = E[q] + w8^q O[q], X[q+4] = E[q] - w8^q O[q]; E, O = DFT4 of even / odd samples.
-template <int S>
-__device__ __forceinline__ void dft8(float2* x) {
+// X[q] = E[q] + w8^q O[q], X[q+4] = E[q] - w8^q O[q]; E, O = DFT4 of even / odd samples, with
+// w8 = h (1 + S i), w8^2 = S i, w8^3 = h (-1 + S i).
+template <int S, class V>
+__device__ __forceinline__ void dft8(V* x) {
   const float h = 0.70710678118654752440f;
-  float2 e[4] = {x[0], x[2], x[4], x[6]};
-  float2 o[4] = {x[1], x[3], x[5], x[7]};
+  V e[4] = {x[0], x[2], x[4], x[6]};
+  V o[4] = {x[1], x[3], x[5], x[7]};
   dft4<S>(e);
   dft4<S>(o);
-  float2 t1 = make_float2(h * (o[1].x - S * o[1].y), h * (o[1].y + S * o[1].x));   // w8^1 = h (1 + S i)
-  float2 t2 = cmul_i<S>(o[2]);                                                     // w8^2 = S i
-  float2 t3 = make_float2(h * (-o[3].x - S * o[3].y), h * (-o[3].y + S * o[3].x)); // w8^3 = h (-1 + S i)
+  const V t1 = cadd_i<S>(o[1], o[1]);    // (1 + S i) o
+  const V t3 = cadd_i<-S>(o[3], o[3]);   // (1 - S i) o = -(-1 + S i) o
   x[0] = cadd(e[0], o[0]);
   x[4] = csub(e[0], o[0]);
-  x[1] = cadd(e[1], t1);
-  x[5] = csub(e[1], t1);
-  x[2] = cadd(e[2], t2);
-  x[6] = csub(e[2], t2);
-  x[3] = cadd(e[3], t3);
-  x[7] = csub(e[3], t3);
+  x[1] = cfma(h, t1, e[1]);
+  x[5] = cfma(-h, t1, e[1]);
+  x[2] = cadd_i<S>(e[2], o[2]);
+  x[6] = cadd_i<-S>(e[2], o[2]);
+  x[3] = cfma(-h, t3, e[3]);
+  x[7] = cfma(h, t3, e[3]);
 }
 
-template <int S>
-__device__ __forceinline__ void dft16(float2* x) {
+template <int S, class V>
+__device__ __forceinline__ void dft16(V* x) {
   // cos(q pi / 8), sin(q pi / 8), q = 0..7
   const float c[8] = {1.0f, 0.92387953251128675613f, 0.70710678118654752440f, 0.38268343236508977173f,
                       0.0f, -0.38268343236508977173f, -0.70710678118654752440f, -0.92387953251128675613f};
   const float s[8] = {0.0f, 0.38268343236508977173f, 0.70710678118654752440f, 0.92387953251128675613f,
                       1.0f, 0.92387953251128675613f, 0.70710678118654752440f, 0.38268343236508977173f};
-  float2 e[8], o[8];
+  V e[8], o[8];
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
     e[i] = x[2 * i];
@@ -173,53 +236,61 @@ __device__ __forceinline__ void dft16(float2* x) {
   dft8<S>(o);
 #pragma unroll
   for (int q = 0; q < 8; ++q) {
-    float2 t = (q == 0) ? o[0] : cmul(o[q], make_float2(c[q], S * s[q]));
-    x[q] = cadd(e[q], t);
-    x[q + 8] = csub(e[q], t);
+    if (q == 4) {
+      x[4] = cadd_i<S>(e[4], o[4]);
+      x[12] = cadd_i<-S>(e[4], o[4]);
+    } else if (q == 2 || q == 6) {   // w = h (+-1 + S i)
+      const V t = q == 2 ? cadd_i<S>(o[2], o[2]) : cadd_i<-S>(o[6], o[6]);
+      const float h = q == 2 ? 0.70710678118654752440f : -0.70710678118654752440f;
+      x[q] = cfma(h, t, e[q]);
+      x[q + 8] = cfma(-h, t, e[q]);
+    } else {
+      const V t = (q == 0) ? o[0] : cmul(o[q], make_float2(c[q], S * s[q]));
+      x[q] = cadd(e[q], t);
+      x[q + 8] = csub(e[q], t);
+    }
   }
 }
 
 // DFT_3: X0 = x0 + x1 + x2, X1,2 = x0 - (x1 + x2)/2 +- S i (sqrt(3)/2)(x1 - x2)
-template <int S>
-__device__ __forceinline__ void dft3(float2* x) {
+template <int S, class V>
+__device__ __forceinline__ void dft3(V* x) {
   const float h = 0.86602540378443864676f;   // sin(2 pi / 3)
-  const float2 t1 = cadd(x[1], x[2]), t2 = csub(x[1], x[2]);
-  const float2 m = make_float2(fmaf(-0.5f, t1.x, x[0].x), fmaf(-0.5f, t1.y, x[0].y));
-  const float2 u = make_float2(-S * h * t2.y, S * h * t2.x);
+  const V t1 = cadd(x[1], x[2]), u = cscale(csub(x[1], x[2]), h);
+  const V m = cfma(-0.5f, t1, x[0]);
   x[0] = cadd(x[0], t1);
-  x[1] = cadd(m, u);
-  x[2] = csub(m, u);
+  x[1] = cadd_i<S>(m, u);
+  x[2] = cadd_i<-S>(m, u);
 }
 
 // DFT_5 by the symmetric pairs a_n = x_n + x_(5-n), b_n = x_n - x_(5-n) (n = 1, 2), with
 // c_q = cos(2 pi q / 5), s_q = sin(2 pi q / 5):
 //   X_1,4 = x0 + c1 a1 + c2 a2 +- S i (s1 b1 + s2 b2),  X_2,3 = x0 + c2 a1 + c1 a2 +- S i (s2 b1 - s1 b2)
-template <int S>
-__device__ __forceinline__ void dft5(float2* x) {
+template <int S, class V>
+__device__ __forceinline__ void dft5(V* x) {
   const float c1 = 0.30901699437494742410f, c2 = -0.80901699437494742410f;
   const float s1 = 0.95105651629515357212f, s2 = 0.58778525229247312917f;
-  const float2 a1 = cadd(x[1], x[4]), b1 = csub(x[1], x[4]);
-  const float2 a2 = cadd(x[2], x[3]), b2 = csub(x[2], x[3]);
-  const float2 p1 = make_float2(x[0].x + c1 * a1.x + c2 * a2.x, x[0].y + c1 * a1.y + c2 * a2.y);
-  const float2 p2 = make_float2(x[0].x + c2 * a1.x + c1 * a2.x, x[0].y + c2 * a1.y + c1 * a2.y);
-  const float2 q1 = make_float2(s1 * b1.x + s2 * b2.x, s1 * b1.y + s2 * b2.y);   // times S i below
-  const float2 q2 = make_float2(s2 * b1.x - s1 * b2.x, s2 * b1.y - s1 * b2.y);
-  const float2 u1 = make_float2(-S * q1.y, S * q1.x), u2 = make_float2(-S * q2.y, S * q2.x);
+  const V a1 = cadd(x[1], x[4]), b1 = csub(x[1], x[4]);
+  const V a2 = cadd(x[2], x[3]), b2 = csub(x[2], x[3]);
+  const V p1 = cfma(c2, a2, cfma(c1, a1, x[0]));
+  const V p2 = cfma(c1, a2, cfma(c2, a1, x[0]));
+  const V q1 = cfma(s2, b2, cscale(b1, s1));   // times S i below
+  const V q2 = cfma(-s1, b2, cscale(b1, s2));
   x[0] = cadd(x[0], cadd(a1, a2));
-  x[1] = cadd(p1, u1);
-  x[4] = csub(p1, u1);
-  x[2] = cadd(p2, u2);
-  x[3] = csub(p2, u2);
+  x[1] = cadd_i<S>(p1, q1);
+  x[4] = cadd_i<-S>(p1, q1);
+  x[2] = cadd_i<S>(p2, q2);
+  x[3] = cadd_i<-S>(p2, q2);
 }
 
-template <int R, int S>
-__device__ __forceinline__ void dft(float2* x) {
+template <int R, int S, class V>
+__device__ __forceinline__ void dft(V* x) {
   if constexpr (R == 3) {
     dft3<S>(x);
   } else if constexpr (R == 5) {
     dft5<S>(x);
   } else if constexpr (R == 2) {
-    float2 t = x[0];
+    const V t = x[0];
     x[0] = cadd(t, x[1]);
     x[1] = csub(t, x[1]);
   } else if constexpr (R == 4) {
@@ -246,13 +317,13 @@ __device__ __forceinline__ float2 wr(int n) {
 //   X[2m] = DFT_H(x)[m],  X[2m+1] = DFT_H(x[n] w_R^n)[m],  w_R = exp(S 2 pi i / R).
 // The first pass of a transform whose upper half is zero padding (Ns = 1) needs no twiddles, so
 // this is the whole butterfly there.
-template <int R, int S>
-__device__ __forceinline__ void dft_half_in(float2* x) {
+template <int R, int S, class V>
+__device__ __forceinline__ void dft_half_in(V* x) {
   constexpr int H = R / 2;
   if constexpr (H == 1) {
     x[1] = x[0];
   } else {
-    float2 e[H], o[H];
+    V e[H], o[H];
 #pragma unroll
     for (int n = 0; n < H; ++n) {
       e[n] = x[n];
@@ -271,13 +342,13 @@ __device__ __forceinline__ void dft_half_in(float2* x) {
 // The first R/2 outputs of DFT_R (sign S) of x: X[q] = E[q] + w_R^q O[q], q < R/2, with E, O the
 // DFT_(R/2) of the even and odd entries (the first half of dft16's combination); x[R/2, R) are
 // left undefined. The last adjoint pass of a cropped transform (Ns = 1) keeps only these.
-template <int R, int S>
-__device__ __forceinline__ void dft_half_out(float2* x) {
+template <int R, int S, class V>
+__device__ __forceinline__ void dft_half_out(V* x) {
   constexpr int H = R / 2;
   if constexpr (H == 1) {
     x[0] = cadd(x[0], x[1]);
   } else {
-    float2 e[H], o[H];
+    V e[H], o[H];
 #pragma unroll
     for (int i = 0; i < H; ++i) {
       e[i] = x[2 * i];
@@ -293,8 +364,8 @@ __device__ __forceinline__ void dft_half_out(float2* x) {
 // v[r] *= exp(S 2 pi i r k / (Ns R)) for r in [1, R): loads w, w^2, w^4, w^8 and forms each
 // other power right before use (w^3 = w w^2, w^(8+r) = w^r w^8, ...), so at most the base
 // powers and one product are live next to the data.
-template <int S, int R, int Ns>
-__device__ __forceinline__ void apply_twiddles(float2* v, int k, const float2* __restrict__ tw) {
+template <int S, int R, int Ns, class V>
+__device__ __forceinline__ void apply_twiddles(V* v, int k, const float2* __restrict__ tw) {
   constexpr int NR = Ns * R;   // w = E_NR, and w^r = E_(NR / r) at the same k < Ns
   const float2 w1 = twiddle_at<S>(tw, NR, k);
   v[1] = cmul(v[1], w1);
@@ -326,8 +397,8 @@ __device__ __forceinline__ void apply_twiddles(float2* v, int k, const float2* _
 }
 
 // Forward butterfly: twiddle, then DFT. Adjoint butterfly: DFT, then twiddle.
-template <int S, int R, int Ns, bool ADJ>
-__device__ __forceinline__ void butterfly(float2* v, int k, const float2* __restrict__ tw) {
+template <int S, int R, int Ns, bool ADJ, class V>
+__device__ __forceinline__ void butterfly(V* v, int k, const float2* __restrict__ tw) {
   if constexpr (!ADJ) {
     if constexpr (Ns > 1) apply_twiddles<S, R, Ns>(v, k, tw);
     dft<R, S>(v);
@@ -353,7 +424,7 @@ __device__ __forceinline__ void stockham_pass(const float2* __restrict__ tw, LD 
   constexpr int NB = (GBD_E + R - 1) / R;   // butterflies per thread (radix 3, 5: the last may be past the end)
   constexpr int T = LINES * L / GBD_E;
   constexpr int NBUT = LINES * LR;
-  float2 v[NB][R];
+  decltype(ld(0, 0)) v[NB][R];   // float2 or cpair
   int bl[NB], bj[NB];
 #pragma unroll
   for (int i = 0; i < NB; ++i) {
@@ -400,8 +471,8 @@ __device__ __forceinline__ void stockham_pass(const float2* __restrict__ tw, LD 
 // HALF (the Ns = 1 pass, even R): forward, the upper half of each line is zero -- only the
 // inputs r < R/2 are loaded and the butterfly is dft_half_in; adjoint, only the lower half of the
 // output is kept -- dft_half_out and the stores q < R/2.
-template <int S, bool ADJ, int L, int R, int Ns, int LINES, bool LF, int LS, bool HALF = false>
-__device__ __forceinline__ void stockham_pass_sm(float2* sm, const float2* __restrict__ tw) {
+template <int S, bool ADJ, int L, int R, int Ns, int LINES, bool LF, int LS, bool HALF = false, class V>
+__device__ __forceinline__ void stockham_pass_sm(V* sm, const float2* __restrict__ tw) {
   static_assert(R % 2 == 0 || Ns == 1, "an odd radix is the Ns = 1 pass");
   static_assert(!HALF || (Ns == 1 && R % 2 == 0), "the half transforms are the Ns = 1 pass of an even radix");
   constexpr int LR = L / R;
@@ -412,7 +483,7 @@ __device__ __forceinline__ void stockham_pass_sm(float2* sm, const float2* __res
   constexpr bool SCA_CONST = (Ns % 16 == 0) || (Ns == 1 && R == 16);
   constexpr int NAT_STRIDE = LR + LR / 16;
   constexpr int SCA_STRIDE = (Ns == 1) ? 1 : Ns + Ns / 16;
-  float2 v[NB][R];
+  V v[NB][R];
   int nat0[NB], sca0[NB], bj[NB];
 #pragma unroll
   for (int i = 0; i < NB; ++i) {

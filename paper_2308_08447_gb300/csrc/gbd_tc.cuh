@@ -232,8 +232,8 @@ __device__ __forceinline__ void pass_any(const float2* __restrict__ tw, LD ld, S
     stockham_pass<S, ADJ, L, R, Ns, LINES, LF, SYNC_MID, HALF>(tw, ld, st);
 }
 
-template <int PREC, int S, bool ADJ, int L, int R, int Ns, int LINES, bool LF, int LS>
-__device__ __forceinline__ void pass_sm_any(float2* sm, const float2* __restrict__ tw) {
+template <int PREC, int S, bool ADJ, int L, int R, int Ns, int LINES, bool LF, int LS, class V>
+__device__ __forceinline__ void pass_sm_any(V* sm, const float2* __restrict__ tw) {
   if constexpr (PREC != 0 && R == 16) {
     auto ld = [&](int line, int i) { return sm[line * LS + pad(i)]; };
     auto st = [&](int line, int i, float2 v) { sm[line * LS + pad(i)] = v; };
@@ -245,8 +245,8 @@ __device__ __forceinline__ void pass_sm_any(float2* sm, const float2* __restrict
 
 // Passes [P, PEND) of the forward chain (sign S) in place in shared memory; LS is the
 // caller's line stride in float2 units.
-template <int S, int L, bool CONV, int LINES, bool LF, int LS, int P, int PEND, int PREC = 0>
-__device__ __forceinline__ void fwd_passes_smem(float2* sm, const float2* __restrict__ tw) {
+template <int S, int L, bool CONV, int LINES, bool LF, int LS, int P, int PEND, int PREC = 0, class V>
+__device__ __forceinline__ void fwd_passes_smem(V* sm, const float2* __restrict__ tw) {
   if constexpr (P < PEND) {
     constexpr int R = radix_at(L, CONV, P);
     constexpr int Ns = ns_at(L, CONV, P);
@@ -257,8 +257,8 @@ __device__ __forceinline__ void fwd_passes_smem(float2* sm, const float2* __rest
 }
 
 // Adjoint passes P-1 down to PEND (inclusive) in place in shared memory.
-template <int S, int L, bool CONV, int LINES, bool LF, int LS, int P, int PEND, int PREC = 0>
-__device__ __forceinline__ void adj_passes_smem(float2* sm, const float2* __restrict__ tw) {
+template <int S, int L, bool CONV, int LINES, bool LF, int LS, int P, int PEND, int PREC = 0, class V>
+__device__ __forceinline__ void adj_passes_smem(V* sm, const float2* __restrict__ tw) {
   if constexpr (P > PEND) {
     constexpr int R = radix_at(L, CONV, P - 1);
     constexpr int Ns = ns_at(L, CONV, P - 1);
