@@ -370,7 +370,7 @@ static void enqueue_conv(gbd_mesh* m, cudaStream_t st) {
     timed(m, GBD_PASS_FILM_CONV, st, [&] { gbd::launch_film_conv(m->p.var_film, m->p.prec, a, m->tw, st); });
     return;
   }
-  a.K3 = static_cast<const float*>(m->K);
+  a.K3 = static_cast<const float2*>(m->K);
   if (p.ny > 1) {
     a.lines_total = 3LL * p.nz * p.Hx;
     a.src = m->S;
@@ -702,14 +702,15 @@ static gbd_status upload_spectrum(gbd_mesh* m, const std::vector<double>& spec, 
         for (int c = 0; c < 4; ++c)
           packed[((size_t)kx * p.Ky + ky) * 4 + c] = (float)spec[c * comp + (size_t)ky * p.Hx + kx];
   } else {
-    // [kz][kx][ky] x (xx, yy, zz, xy, xz, yz): the z convolution's lanes take consecutive
-    // (kx, ky) columns at one kz, so they read consecutive entries
+    // [kz][pair][kx][ky] x (xx, yy), (zz, xy), (xz, yz): the z convolution's lanes take consecutive
+    // (kx, ky) columns at one kz, so each of its loads reads consecutive 8-byte entries
     for (int kz = 0; kz < p.Kz; ++kz)
-      for (int kx = 0; kx < p.Hx; ++kx)
-        for (int ky = 0; ky < p.Ky; ++ky)
-          for (int c = 0; c < 6; ++c)
-            packed[(((size_t)kz * p.Hx + kx) * p.Ky + ky) * 6 + c] =
-                (float)spec[c * comp + (size_t)kz * plane + (size_t)ky * p.Hx + kx];
+      for (int i = 0; i < 3; ++i)
+        for (int kx = 0; kx < p.Hx; ++kx)
+          for (int ky = 0; ky < p.Ky; ++ky)
+            for (int c = 0; c < 2; ++c)
+              packed[((((size_t)kz * 3 + i) * p.Hx + kx) * p.Ky + ky) * 2 + c] =
+                  (float)spec[(2 * i + c) * comp + (size_t)kz * plane + (size_t)ky * p.Hx + kx];
   }
   cudaError_t e = cudaMemcpyAsync(m->K, packed.data(), p.bytes_K, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
@@ -1382,7 +1383,7 @@ void enqueue_conv_on(const gbd_mesh* m, float2* S, float2* T, cudaStream_t st) {
     gbd::launch_film_conv(m->p.var_film, m->p.prec, a, m->tw, st);
     return;
   }
-  a.K3 = static_cast<const float*>(m->K);
+  a.K3 = static_cast<const float2*>(m->K);
   if (p.ny > 1) {
     a.lines_total = 3LL * p.nz * p.Hx;
     a.src = S;
@@ -1736,7 +1737,7 @@ extern "C" gbd_status gbd_mesh_autotune(gbd_mesh* m, void* stream) {
     ca.Kf = static_cast<const float4*>(m->K);
     e = pick(1, [&](int v) { gbd::launch_film_conv(v, p.prec, ca, m->tw, st); });
   } else if (e == cudaSuccess) {
-    ca.K3 = static_cast<const float*>(m->K);
+    ca.K3 = static_cast<const float2*>(m->K);
     if (p.ny > 1) {
       ca.lines_total = 3LL * p.nz * p.Hx;
       ca.src = m->S;

@@ -21,17 +21,21 @@ static bool z_dispatch(int Pz, int var, int prec, const ColArgs* a, const float2
 }
 
 bool launch_film_conv(int var, int prec, const ColArgs& a, const float2* tw, cudaStream_t st) {
+  prec = stage_prec(prec, a.Py, true);
   if (mixed_len(a.Py)) return prec == 0 && film_dispatch_mixed(a.Py, &a, tw, st);
   return film_dispatch(a.Py, var, prec, &a, tw, st);
 }
 bool prepare_film_conv(int Py, int prec) {
+  prec = stage_prec(prec, Py, true);
   if (mixed_len(Py)) return prec <= 0 && film_dispatch_mixed(Py, nullptr, nullptr, nullptr);
   return film_dispatch(Py, -1, prec, nullptr, nullptr, nullptr);
 }
 
 bool launch_z_conv(int var, int prec, const ColArgs& a, const float2* tw, cudaStream_t st) {
-  return z_dispatch(a.Pz, var, prec, &a, tw, st);
+  return z_dispatch(a.Pz, var, stage_prec(prec, a.Pz, true), &a, tw, st);
 }
-bool prepare_z_conv(int Pz, int prec) { return z_dispatch(Pz, -1, prec, nullptr, nullptr, nullptr); }
+bool prepare_z_conv(int Pz, int prec) {
+  return z_dispatch(Pz, -1, stage_prec(prec, Pz, true), nullptr, nullptr, nullptr);
+}
 
 }  // namespace gbd

@@ -195,10 +195,14 @@ __global__ void __launch_bounds__(3 * C_ * L / GBD_E,
 // 3D z convolution: one block = W consecutive columns q = kx Py + ky of the y spectrum T,
 // three components each (lines c W + w); the z FFT reads the nz planes (zero padding above),
 // the product couples the three components, and the adjoint z FFT writes back the nz planes.
+// Blocks per SM of the z convolution: FP32 at 24 warps (80 registers for the 48 values of a fused item)
+__host__ __device__ constexpr int zconv_blocks(int T, int prec) {
+  const int w = (T + 31) / 32;
+  return prec ? min_blocks(T) : 24 / w < 1 ? 1 : 24 / w;
+}
 template <int L, int W_, int PREC>
-__global__ void __launch_bounds__(3 * W_ * L / GBD_E,
-                                  PREC == 0 ? min_blocks_film(3 * W_ * L / GBD_E) : min_blocks(3 * W_ * L / GBD_E))
-    z_conv_kernel(ColArgs a, const float2* __restrict__ tw) {
+__global__ void __launch_bounds__(3 * W_ * L / GBD_E, zconv_blocks(3 * W_ * L / GBD_E, PREC))
+    z_conv_kernel(const __grid_constant__ ColArgs a, const float2* __restrict__ tw) {
   constexpr int W = W_;
   constexpr int LINES = 3 * W;
   constexpr int T = LINES * L / GBD_E;
@@ -209,6 +213,24 @@ __global__ void __launch_bounds__(3 * W_ * L / GBD_E,
   constexpr int LR = L / RL;
   extern __shared__ float2 sm[];
   const long long q0 = (long long)blockIdx.x * W;
+  // FP32 with two or more passes: the block's kernel columns [kz][pair][w], kz <= L / 2, are copied
+  // into shared memory behind the lines while the forward transform runs (they do not depend on the
+  // preceding launch, so ahead of the wait for it)
+  constexpr bool SK = PREC == 0 && NP > 1;
+  float2* sK = sm + LINES * LS;
+  if constexpr (SK) {
+    static_assert(T % W == 0, "a thread copies one column");
+    const int w = threadIdx.x % W, q = (int)q0 + w;
+    if (q < (int)a.Q) {
+      const int kx = q / a.Pyq, ky = q - kx * a.Pyq, KYs = a.Py / 2 + 1;
+      const int kyp = (a.Py > 1 && ky > a.Py / 2) ? a.Py - ky : ky;
+      const long long kpl = (long long)a.Hx * KYs;
+      const float2* src = a.K3 + (long long)kx * KYs + kyp;
+      for (int t = threadIdx.x / W; t < 3 * (L / 2 + 1); t += T / W) cp_async8(sK + t * W + w, src + t * kpl);
+    }
+    cp_async_commit();
+  }
+  pdl_wait_then_release();
   const int nz = a.nz;
   const long long Q = a.Q;
   const int Qi = (int)Q;   // Hx Py <= 4097 * 4096: a plane offset z Q fits in 32-bit int arithmetic
@@ -228,38 +250,41 @@ __global__ void __launch_bounds__(3 * W_ * L / GBD_E,
   auto run_fused = [&](auto ld, auto st) {
     for (int it = threadIdx.x; it < W * LR; it += T) {
       const int w = it % W, j = it / W;
-      const long long q = q0 + w;
-      const int kx = (int)(q / Pyq);
-      const int ky = (int)(q - (long long)kx * Pyq);
-      int kyp = ky;
-      float sy = 1.f;
-      if (Py > 1 && ky > Py / 2) {
-        kyp = Py - ky;
-        sy = -1.f;
-      }
-      const float* kbase = a.K3 + ((long long)kx * KY + kyp) * 6;   // + kz' Hx KY 6
-      auto mul = [&](int kz, float2& m0, float2& m1, float2& m2) {
-        if (q >= Q) return;
-        int kzp = kz;
-        float sz = 1.f;
-        if (kz > L / 2) {
-          kzp = L - kz;
-          sz = -1.f;
-        }
-        const float* kp = kbase + (long long)kzp * a.Hx * KY * 6;
-        const float2 k01 = __ldg(reinterpret_cast<const float2*>(kp));
-        const float2 k23 = __ldg(reinterpret_cast<const float2*>(kp + 2));
-        const float2 k45 = __ldg(reinterpret_cast<const float2*>(kp + 4));
+      const int q = (int)q0 + w;
+      if (q >= Q) continue;   // past the last column: nothing of it is kept
+      const int kx = q / Pyq, ky = q - kx * Pyq;   // q < Q = Hx Py fits in int: 32-bit division
+      const bool up = Py > 1 && ky > Py / 2;
+      const float sy = up ? -1.f : 1.f;
+      const long long kpl = SK ? W : (long long)a.Hx * KY;      // between the pairs of one kz
+      const float2* kcol = SK ? sK + w : a.K3 + (long long)kx * KY + (up ? Py - ky : ky);
+      float2 v[3][RL];
+#pragma unroll
+      for (int c = 0; c < 3; ++c)
+#pragma unroll
+        for (int r = 0; r < RL; ++r) v[c][r] = ld(w + c * W, j + r * LR);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) butterfly<-1, RL, NSL, false>(v[c], j, tw);
+#pragma unroll
+      for (int r = 0; r < RL; ++r) {
+        // frequency kz = j + r L/R, stored at kz or, above L/2 (r >= R/2 but for kz = L/2), at L - kz
+        // with the z-odd components negated
+        const int kz = r < RL / 2 || RL == 1 ? j + r * LR : L - j - r * LR;
+        const float sz = r < RL / 2 || RL == 1 || (r == RL / 2 && j == 0) ? 1.f : -1.f;
+        const float2* kp = kcol + kz * 3 * kpl;
+        const float2 k01 = kp[0], k23 = kp[kpl], k45 = kp[2 * kpl];
         const float kxx = k01.x, kyy = k01.y, kzz = k23.x;
         const float kxy = sy * k23.y, kxz = sz * k45.x, kyz = sy * sz * k45.y;
-        const float2 h0 = make_float2(kxx * m0.x + kxy * m1.x + kxz * m2.x, kxx * m0.y + kxy * m1.y + kxz * m2.y);
-        const float2 h1 = make_float2(kxy * m0.x + kyy * m1.x + kyz * m2.x, kxy * m0.y + kyy * m1.y + kyz * m2.y);
-        const float2 h2 = make_float2(kxz * m0.x + kyz * m1.x + kzz * m2.x, kxz * m0.y + kyz * m1.y + kzz * m2.y);
-        m0 = h0;
-        m1 = h1;
-        m2 = h2;
-      };
-      fused_item<L, RL, NSL>(w, W, j, tw, ld, st, mul);
+        const float2 m0 = v[0][r], m1 = v[1][r], m2 = v[2][r];
+        v[0][r] = make_float2(kxx * m0.x + kxy * m1.x + kxz * m2.x, kxx * m0.y + kxy * m1.y + kxz * m2.y);
+        v[1][r] = make_float2(kxy * m0.x + kyy * m1.x + kyz * m2.x, kxy * m0.y + kyy * m1.y + kyz * m2.y);
+        v[2][r] = make_float2(kxz * m0.x + kyz * m1.x + kzz * m2.x, kxz * m0.y + kyz * m1.y + kzz * m2.y);
+      }
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        butterfly<1, RL, NSL, true>(v[c], j, tw);
+#pragma unroll
+        for (int r = 0; r < RL; ++r) st(w + c * W, j + r * LR, v[c][r]);
+      }
     }
   };
   if constexpr (NP == 1) {
@@ -294,76 +319,84 @@ __global__ void __launch_bounds__(3 * W_ * L / GBD_E,
     }
     __syncthreads();
     fwd_passes_smem<-1, L, true, LINES, true, LS, 1, NP - 1, PREC>(sm, tw);
-    // The last forward pass, the product and the first adjoint pass as three in-place phases
-    // over all threads: the last pass (Ns R = L) leaves frequency j + q L/R at the position
-    // it read, so each phase touches only its own items' positions.
-    // T is a multiple of LINES, so a thread keeps one line through its 16 / RL items, and with
-    // LR a multiple of 16 an item's RL elements sit at pad(j) + r (LR + LR/16): one base address
-    // per item and compile-time offsets.
-    static_assert(T % LINES == 0 && (LINES * LR) % T == 0, "z convolution: items per thread");
-    auto last_pass = [&](auto adj) {
-      constexpr bool ADJ = decltype(adj)::value;
-      constexpr int NI = LINES * LR / T;
-      constexpr bool NAT = (LR % 16 == 0);
-      constexpr int STRIDE = LR + LR / 16;
-      const int line = threadIdx.x % LINES;
-      const int j0 = threadIdx.x / LINES;
-#pragma unroll
-      for (int i = 0; i < NI; ++i) {
-        const int j = j0 + i * (T / LINES);
-        float2* lp = sm + line * LS + (NAT ? pad(j) : 0);
-        float2 v[RL];
-#pragma unroll
-        for (int r = 0; r < RL; ++r) v[r] = NAT ? lp[r * STRIDE] : lp[pad(j + r * LR)];
-        butterfly<ADJ ? 1 : -1, RL, NSL, ADJ>(v, j, tw);
-#pragma unroll
-        for (int r = 0; r < RL; ++r) {
-          if (NAT)
-            lp[r * STRIDE] = v[r];
-          else
-            lp[pad(j + r * LR)] = v[r];
+    if constexpr (SK) {
+      // The last forward pass, the product and the first adjoint pass in registers, one thread per
+      // (column w, butterfly j) with the three components: frequency j + q L/R stays at the position
+      // it was read from, so an item touches only its own positions.
+      cp_async_wait<0>();
+      __syncthreads();
+      run_fused(sld, sst);
+      __syncthreads();
+    } else {
+      // The last forward pass, the product and the first adjoint pass as three in-place phases
+      // over all threads: the last pass (Ns R = L) leaves frequency j + q L/R at the position
+      // it read, so each phase touches only its own items' positions.
+      // T is a multiple of LINES, so a thread keeps one line through its 16 / RL items, and with
+      // LR a multiple of 16 an item's RL elements sit at pad(j) + r (LR + LR/16): one base address
+      // per item and compile-time offsets.
+      static_assert(T % LINES == 0 && (LINES * LR) % T == 0, "z convolution: items per thread");
+      auto last_pass = [&](auto adj) {
+        constexpr bool ADJ = decltype(adj)::value;
+        constexpr int NI = LINES * LR / T;
+        constexpr bool NAT = (LR % 16 == 0);
+        constexpr int STRIDE = LR + LR / 16;
+        const int line = threadIdx.x % LINES;
+        const int j0 = threadIdx.x / LINES;
+  #pragma unroll
+        for (int i = 0; i < NI; ++i) {
+          const int j = j0 + i * (T / LINES);
+          float2* lp = sm + line * LS + (NAT ? pad(j) : 0);
+          float2 v[RL];
+  #pragma unroll
+          for (int r = 0; r < RL; ++r) v[r] = NAT ? lp[r * STRIDE] : lp[pad(j + r * LR)];
+          butterfly<ADJ ? 1 : -1, RL, NSL, ADJ>(v, j, tw);
+  #pragma unroll
+          for (int r = 0; r < RL; ++r) {
+            if (NAT)
+              lp[r * STRIDE] = v[r];
+            else
+              lp[pad(j + r * LR)] = v[r];
+          }
         }
-      }
-    };
-    last_pass(std::false_type());
-    __syncthreads();
-    // product at (column w, frequencies kz and Pz - kz): consecutive lanes take consecutive
-    // columns; T is a multiple of W, so each thread keeps one column and its (kx, ky) are worked
-    // out once. The stored kernel at kz' = kz serves both kz and Pz - kz (the latter with the
-    // z-odd components xz, yz negated), so an item loads it once for the pair.
-    static_assert(T % W == 0, "a thread's product items share one column");
-    const int w = threadIdx.x % W;
-    const long long q = q0 + w;
-    const int kx = (int)q / Pyq;   // q < Q = Hx Py fits in int: 32-bit division
-    const int ky = (int)q - kx * Pyq;
-    int kyp = ky;
-    float sy = 1.f;
-    if (Py > 1 && ky > Py / 2) {
-      kyp = Py - ky;
-      sy = -1.f;
-    }
-    const float* kcol = a.K3 + ((long long)kx * KY + kyp) * 6;
-    const long long kzs = (long long)a.Hx * KY * 6;      // kernel stride between kz planes
-    for (int kz = threadIdx.x / W; kz <= L / 2 && q < Q; kz += T / W) {
-      const float* kp = kcol + kz * kzs;
-      const float2 k01 = __ldg(reinterpret_cast<const float2*>(kp));
-      const float2 k23 = __ldg(reinterpret_cast<const float2*>(kp + 2));
-      const float2 k45 = __ldg(reinterpret_cast<const float2*>(kp + 4));
-      const float kxx = k01.x, kyy = k01.y, kzz = k23.x;
-      const float kxy = sy * k23.y, kxz0 = k45.x, kyz0 = sy * k45.y;
-      auto apply = [&](int z, float sz) {
-        const float kxz = sz * kxz0, kyz = sz * kyz0;
-        const float2 m0 = sld(w, z), m1 = sld(W + w, z), m2 = sld(2 * W + w, z);
-        sst(w, z, make_float2(kxx * m0.x + kxy * m1.x + kxz * m2.x, kxx * m0.y + kxy * m1.y + kxz * m2.y));
-        sst(W + w, z, make_float2(kxy * m0.x + kyy * m1.x + kyz * m2.x, kxy * m0.y + kyy * m1.y + kyz * m2.y));
-        sst(2 * W + w, z, make_float2(kxz * m0.x + kyz * m1.x + kzz * m2.x, kxz * m0.y + kyz * m1.y + kzz * m2.y));
       };
-      apply(kz, 1.f);
-      if (kz > 0 && kz < L / 2) apply(L - kz, -1.f);
+      last_pass(std::false_type());
+      __syncthreads();
+      // product at (column w, frequencies kz and Pz - kz): consecutive lanes take consecutive
+      // columns; T is a multiple of W, so each thread keeps one column and its (kx, ky) are worked
+      // out once. The stored kernel at kz' = kz serves both kz and Pz - kz (the latter with the
+      // z-odd components xz, yz negated), so an item loads it once for the pair.
+      static_assert(T % W == 0, "a thread's product items share one column");
+      const int w = threadIdx.x % W;
+      const long long q = q0 + w;
+      const int kx = (int)q / Pyq;   // q < Q = Hx Py fits in int: 32-bit division
+      const int ky = (int)q - kx * Pyq;
+      int kyp = ky;
+      float sy = 1.f;
+      if (Py > 1 && ky > Py / 2) {
+        kyp = Py - ky;
+        sy = -1.f;
+      }
+      const long long kpl = (long long)a.Hx * KY;
+      const float2* kcol = a.K3 + (long long)kx * KY + kyp;
+      for (int kz = threadIdx.x / W; kz <= L / 2 && q < Q; kz += T / W) {
+        const float2* kp = kcol + 3 * kz * kpl;
+        const float2 k01 = __ldg(kp), k23 = __ldg(kp + kpl), k45 = __ldg(kp + 2 * kpl);
+        const float kxx = k01.x, kyy = k01.y, kzz = k23.x;
+        const float kxy = sy * k23.y, kxz0 = k45.x, kyz0 = sy * k45.y;
+        auto apply = [&](int z, float sz) {
+          const float kxz = sz * kxz0, kyz = sz * kyz0;
+          const float2 m0 = sld(w, z), m1 = sld(W + w, z), m2 = sld(2 * W + w, z);
+          sst(w, z, make_float2(kxx * m0.x + kxy * m1.x + kxz * m2.x, kxx * m0.y + kxy * m1.y + kxz * m2.y));
+          sst(W + w, z, make_float2(kxy * m0.x + kyy * m1.x + kyz * m2.x, kxy * m0.y + kyy * m1.y + kyz * m2.y));
+          sst(2 * W + w, z, make_float2(kxz * m0.x + kyz * m1.x + kzz * m2.x, kxz * m0.y + kyz * m1.y + kzz * m2.y));
+        };
+        apply(kz, 1.f);
+        if (kz > 0 && kz < L / 2) apply(L - kz, -1.f);
+      }
+      __syncthreads();
+      last_pass(std::true_type());
+      __syncthreads();
     }
-    __syncthreads();
-    last_pass(std::true_type());
-    __syncthreads();
     adj_passes_smem<1, L, true, LINES, true, LS, NP - 1, 1, PREC>(sm, tw);
     if (FAST && half) {
       const float2* sp = sm + fline * LS + 17 * fj;
@@ -400,9 +433,10 @@ static void film_launch_t(const ColArgs* a, const float2* tw, cudaStream_t st) {
 template <int L, int W, int PREC>
 static void zconv_launch_t(const ColArgs* a, const float2* tw, cudaStream_t st) {
   constexpr int T = 3 * W * L / GBD_E;
-  const size_t smem = (size_t)3 * W * line_stride<L, true>() * sizeof(float2);
+  const size_t kcols = PREC == 0 && npasses(L, true) > 1 ? (size_t)3 * (L / 2 + 1) * W : 0;   // staged kernel columns
+  const size_t smem = ((size_t)3 * W * line_stride<L, true>() + kcols) * sizeof(float2);
   prep(z_conv_kernel<L, W, PREC>, smem);
-  if (a) z_conv_kernel<L, W, PREC><<<(unsigned)((a->Q + W - 1) / W), T, smem, st>>>(*a, tw);
+  if (a) launch_pdl(z_conv_kernel<L, W, PREC>, (unsigned)((a->Q + W - 1) / W), T, smem, st, *a, tw);
 }
 
 // Calls f(std::integral_constant<int, L>) for a transform length L in {1, 4, 8, ..., 4096}
@@ -431,26 +465,48 @@ static bool conv_switch(int L, F f) {
   }
 }
 
+// Launches (a == nullptr: prepares every tile of) the film convolution of length L with the tile of
+// variant var for a's columns.
+template <int L, int PREC>
+static void film_launch_tile(int var, const ColArgs* a, const float2* tw, cudaStream_t st) {
+  constexpr int V0 = film_cols(L, 0), V1 = film_cols(L, 1);
+  constexpr int S0 = film_cols_small(L, PREC, 0), S1 = film_cols_small(L, PREC, 1);
+  const int c = a ? pick_tile(a->Hx, var == 0 ? V0 : V1, V0, S0, S1) : 0;
+  if (!a || c == V0) film_launch_t<L, V0, PREC>(a, tw, st);
+  if constexpr (V1 != V0)
+    if (!a || c == V1) film_launch_t<L, V1, PREC>(a, tw, st);
+  if constexpr (S0 > 0)
+    if (!a || c == S0) film_launch_t<L, S0, PREC>(a, tw, st);
+  if constexpr (S1 > 0)
+    if (!a || c == S1) film_launch_t<L, S1, PREC>(a, tw, st);
+}
+template <int L, int PREC>
+static void zconv_launch_tile(int var, const ColArgs* a, const float2* tw, cudaStream_t st) {
+  constexpr int V0 = zconv_cols(L, 0), V1 = zconv_cols(L, 1);
+  constexpr int S0 = zconv_cols_small(L, PREC, 0), S1 = zconv_cols_small(L, PREC, 1);
+  const int w = a ? pick_tile(a->Q, var == 0 ? V0 : V1, V1, S0, S1) : 0;
+  if (!a || w == V0) zconv_launch_t<L, V0, PREC>(a, tw, st);
+  if constexpr (V1 != V0)
+    if (!a || w == V1) zconv_launch_t<L, V1, PREC>(a, tw, st);
+  if constexpr (S0 > 0)
+    if (!a || w == S0) zconv_launch_t<L, S0, PREC>(a, tw, st);
+  if constexpr (S1 > 0)
+    if (!a || w == S1) zconv_launch_t<L, S1, PREC>(a, tw, st);
+}
+
 // Launch (a == nullptr: prepare) the film / z convolution of precision PREC for transform
-// length Py / Pz, tile variant var (both when var < 0). Explicitly instantiated once per
-// precision, each in its own translation unit, so the units build in parallel.
+// length Py / Pz, tile variant var. Explicitly instantiated once per precision, each in its own
+// translation unit, so the units build in parallel.
 template <int PREC>
 bool film_dispatch_p(int Py, int var, const ColArgs* a, const float2* tw, cudaStream_t st) {
-  return conv_switch(Py, [&](auto l) {
-    constexpr int L = decltype(l)::value;
-    if (var <= 0) film_launch_t<L, film_cols(L, 0), PREC>(a, tw, st);
-    if (var != 0) film_launch_t<L, film_cols(L, 1), PREC>(a, tw, st);
-  });
+  return conv_switch(Py, [&](auto l) { film_launch_tile<decltype(l)::value, PREC>(var, a, tw, st); });
 }
 template <int PREC>
 bool z_dispatch_p(int Pz, int var, const ColArgs* a, const float2* tw, cudaStream_t st) {
   if (Pz < 4) return false;
   return conv_switch(Pz, [&](auto l) {
     constexpr int L = decltype(l)::value;
-    if constexpr (L >= 4) {
-      if (var <= 0) zconv_launch_t<L, zconv_cols(L, 0), PREC>(a, tw, st);
-      if (var != 0) zconv_launch_t<L, zconv_cols(L, 1), PREC>(a, tw, st);
-    }
+    if constexpr (L >= 4) zconv_launch_tile<L, PREC>(var, a, tw, st);
   });
 }
 extern template bool film_dispatch_p<1>(int, int, const ColArgs*, const float2*, cudaStream_t);

@@ -46,6 +46,16 @@ __host__ __device__ constexpr int row_rb(int Lx, int v) {
          : v == 0      ? (Lx >= 2048 ? 1 : 2048 / Lx)
                        : (Lx >= 4096 ? 1 : 4096 / Lx);
 }
+// Smaller row tiles, for meshes whose rows would fill too few of them: the row counts below the
+// variant's that have kernels -- 2 rows (one 16-byte vector of the [kx][y] spectrum) or as many
+// as give a block 48 threads, and four and sixteen times that. The tensor-core passes need whole warps.
+__host__ __device__ constexpr int row_rb_min(int Lx, int prec) {
+  return prec != 0 ? (Lx >= 256 ? 2 : Lx >= 16 ? 512 / Lx : row_rb(Lx, 0))
+                   : (pow2_floor(Lx) >= 128 ? 2 : Lx >= 16 ? 256 / pow2_floor(Lx) : row_rb(Lx, 0));
+}
+__host__ __device__ constexpr int row_rb_small(int Lx, int prec, int i) {   // i = 0, 1, 2 (0: none)
+  return (row_rb_min(Lx, prec) << (2 * i)) < row_rb(Lx, 0) ? row_rb_min(Lx, prec) << (2 * i) : 0;
+}
 // kx columns per film-convolution block (3 lines each)
 __host__ __device__ constexpr int film_cols(int Py, int v) {
   return mixed_len(Py) ? (pow2_floor(Py) >= 1024 ? 1 : 1024 / pow2_floor(Py))
@@ -61,6 +71,34 @@ __host__ __device__ constexpr int ypass_lines(int Py, int v) {
 // (kx, ky) columns per z-convolution block (3 lines each)
 __host__ __device__ constexpr int zconv_cols(int Pz, int v) {
   return v == 0 ? (Pz >= 2048 ? 1 : 2048 / Pz) : (Pz >= 1024 ? 1 : 1024 / Pz);
+}
+
+// Smaller tiles of the same kinds: lines of v = 1 (the z and y passes) or v = 0 (film) over 2 and 4
+// (film and z: 96 and 48 threads per block, y: 64 and 32); the second for FP32 only (the tensor-core
+// passes need whole warps).
+__host__ __device__ constexpr int film_cols_small(int Py, int prec, int i) {
+  return mixed_len(Py) ? (i == 0 ? film_cols(Py, 0) / 2 : film_cols(Py, 0) / 4)
+                       : (Py > 1 && (i == 0 || prec == 0)) ? (1024 / Py) >> (i + 1) : 0;
+}
+__host__ __device__ constexpr int ypass_lines_small(int Py, int i) {
+  return mixed_len(Py) ? (i == 0 ? ypass_lines(Py, 0) / 4 : ypass_lines(Py, 0) / 8) : (2048 / Py) >> (i + 1);
+}
+__host__ __device__ constexpr int zconv_cols_small(int Pz, int prec, int i) {
+  return (i == 0 || prec == 0) ? (1024 / Pz) >> (i + 1) : 0;
+}
+// A launch takes a smaller tile while its own spreads it over fewer blocks than the GPU has SMs. A
+// block takes the same ~10 us on an empty SM whatever its tile, so idle SMs cost in proportion; but
+// twice as many blocks as SMs is already slower where the tile's half sectors and barriers count.
+// RK stage, us, by the number of blocks asked for (none / 152 / 304): 96x64x1 24.3 / 13.5 / 13.5,
+// 480x240x2 45.2 / 39.2 / 39.2, 192x224x8 56.7 / 50.7 / 59.9, 512x256x8 114.9 / 108.3 / 116.3.
+constexpr int kTileBlocks = 152;
+// The tile of a launch over `lines` rows, columns or lines: the variant's tile v, or the largest of
+// the smaller ones s0 > s1 > ... (0: none) that spreads the launch over kTileBlocks blocks.
+inline int pick_tile(long long lines, int v, int s0, int s1, int s2 = 0, int s3 = 0) {
+  int t = v;
+  for (int s : {s0, s1, s2, s3})
+    if (s > 0 && s < t && (lines + t - 1) / t < kTileBlocks) t = s;
+  return t;
 }
 
 struct RowArgs {
@@ -140,8 +178,8 @@ struct ColArgs {
   const float2* src;
   float2* dst;
   const float4* Kf;         // film kernel [Hx][Py/2+1] (xx, yy, zz, xy)
-  const float* K3;          // 3D kernel [Pz/2+1][Hx][Py/2+1][6]
-  long long Q;              // z-conv columns per plane = Hx * Py (Hx when ny == 1)
+  const float2* K3;         // 3D kernel [Pz/2+1][3][Hx][Py/2+1]: (xx, yy), (zz, xy), (xz, yz)
+  long long Q;              // z-conv columns = Hx * Py (Hx when ny == 1)
   int Pyq;                  // y extent of the column index q (Py, or 1 when ny == 1)
 };
 
@@ -186,6 +224,14 @@ bool row_dispatch_mixed(int Lx, int var, const RowArgs* a, const float2* tw, cud
 bool film_dispatch_mixed(int Py, const ColArgs* a, const float2* tw, cudaStream_t st);
 bool ypass_dispatch_mixed(int Py, bool inv, const ColArgs* a, const float2* tw, cudaStream_t st);
 
+// The precision a transform of length L runs in (conv: in a convolution kernel): without a radix-16
+// pass it is the FP32 transform in every precision, and takes the FP32 kernels.
+inline int stage_prec(int prec, int L, bool conv) {
+  if (prec > 0)
+    for (int p = 0; p < npasses(L, conv); ++p)
+      if (radix_at(L, conv, p) == 16) return prec;
+  return prec < 0 ? prec : 0;
+}
 // Set the kernels' shared-memory attribute for both variants of a length without launching
 // (done when a mesh is created, so later launches inside a stream capture need no driver
 // configuration call). Return false for a length without an instantiation.

@@ -42,6 +42,20 @@ static void launch_pdl(void (*k)(P...), unsigned grid, unsigned block, size_t sm
   cudaLaunchKernelEx(&cfg, k, static_cast<A&&>(args)...);
 }
 
+// Asynchronous global -> shared copies (cp.async, 16 or 8 bytes per thread), in commit groups.
+__device__ __forceinline__ unsigned smem_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void cp_async16(void* s, const void* g) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_addr(s)), "l"(g) : "memory");
+}
+__device__ __forceinline__ void cp_async8(void* s, const void* g) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(smem_addr(s)), "l"(g) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
+}
+
 // Raises the dynamic shared-memory limit of kernel k once per (kernel, device). Meshes call
 // this for their kernels when they are created, so launches inside a stream capture find the
 // attribute already set.

@@ -1,5 +1,5 @@
 // Film convolution and 3D y passes for the transform lengths Py = 3 * 2^k and 5 * 2^k (FP32;
-// gbd_fft.cuh), one tile shape each: the y padding of Sec. II at the smallest length
+// gbd_fft.cuh): the y padding of Sec. II at the smallest length
 // >= 2 ny - 1 of the form 2^a 3^b 5^c with b + c <= 1.
 #include "gbd_conv.cuh"
 #include "gbd_ypass.cuh"
@@ -32,7 +32,7 @@ static bool mixed_switch(int L, F f) {
 bool film_dispatch_mixed(int Py, const ColArgs* a, const float2* tw, cudaStream_t st) {
   return mixed_switch(Py, [&](auto l) {
     constexpr int L = decltype(l)::value;
-    film_launch_t<L, film_cols(L, 0), 0>(a, tw, st);
+    film_launch_tile<L, 0>(0, a, tw, st);
   });
 }
 
@@ -40,9 +40,9 @@ bool ypass_dispatch_mixed(int Py, bool inv, const ColArgs* a, const float2* tw, 
   return mixed_switch(Py, [&](auto l) {
     constexpr int L = decltype(l)::value;
     if (inv)
-      ypass_launch_t<L, ypass_lines(L, 0), true, 0>(a, tw, st);
+      ypass_launch_tile<L, true, 0>(0, a, tw, st);
     else
-      ypass_launch_t<L, ypass_lines(L, 0), false, 0>(a, tw, st);
+      ypass_launch_tile<L, false, 0>(0, a, tw, st);
   });
 }
 

@@ -1,7 +1,6 @@
 // x-row kernels for the transform lengths Lx = 3 * 2^k and 5 * 2^k (FP32; gbd_fft.cuh), so that
 // the zero padding of Sec. II can stop at the smallest length 2 Lx >= 2 nx - 1 of the form
-// 2^a 3^b 5^c with b + c <= 1 instead of the next power of two: row_kernel (one tile shape)
-// and the persistent pipelined kernel (gbd_rowpipe.cuh) where it applies.
+// 2^a 3^b 5^c with b + c <= 1 instead of the next power of two: row_kernel and the persistent pipelined kernel (gbd_rowpipe.cuh) where it applies.
 #include "gbd_rowpipe.cuh"
 
 namespace gbd {
@@ -36,7 +35,7 @@ bool row_dispatch_mixed(int Lx, int var, const RowArgs* a, const float2* tw, cud
     pipe_dispatch_with(sw, Lx, -1, nullptr, nullptr, nullptr);
     return mixed_switch(Lx, [&](auto lx) {
       constexpr int LX = decltype(lx)::value;
-      row_launch_t<LX, row_rb(LX, 0), 0>(nullptr, nullptr, nullptr);
+      row_launch_tile<LX, 0>(0, nullptr, nullptr, nullptr);
     });
   }
   if (var >= 2) {
@@ -45,7 +44,7 @@ bool row_dispatch_mixed(int Lx, int var, const RowArgs* a, const float2* tw, cud
   }
   return mixed_switch(Lx, [&](auto lx) {
     constexpr int LX = decltype(lx)::value;
-    row_launch_t<LX, row_rb(LX, 0), 0>(a, tw, st);
+    row_launch_tile<LX, 0>(0, a, tw, st);
   });
 }
 

@@ -85,7 +85,7 @@ __global__ void __launch_bounds__(256) extrap_stage_kernel(const RowArgs a) {
     const long long idx = (long long)row * nx + 2 * xp;
     float hd[2][3], mn[2][3];
     extrap_pair(a, idx, hd);
-    epilogue_pair(a, a.mode, z, y, idx, 2 * xp, threadIdx.x & 31, hd, mn);
+    epilogue_pair<true>(a, a.mode, z, y, idx, 2 * xp, threadIdx.x & 31, hd, mn);
   } else {
     if (i >= a.N) return;
     const int row = (int)(i / nx);

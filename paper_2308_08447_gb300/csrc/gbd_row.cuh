@@ -50,20 +50,6 @@ __device__ __forceinline__ bool mbar_wait(unsigned long long* b, unsigned parity
   }
 }
 
-// Asynchronous global -> shared copies (cp.async, 16 or 8 bytes per thread), in commit groups.
-__device__ __forceinline__ unsigned smem_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void cp_async16(void* s, const void* g) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_addr(s)), "l"(g) : "memory");
-}
-__device__ __forceinline__ void cp_async8(void* s, const void* g) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(smem_addr(s)), "l"(g) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() {
-  asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
-}
-
 // ---------------------------------------------------------------------------------------------
 // x rows: real-to-complex through a half-length complex FFT (Lx = Px / 2).
 // Forward: z[m] = x[2m] + i x[2m+1], Z = FFT_Lx(z), and for k in [0, Lx]
@@ -170,10 +156,11 @@ __device__ __forceinline__ void extrap_cell(const RowArgs& a, long long idx, flo
 }
 
 // Epilogue of the pair of cells (x0, x0 + 1), x0 even, at linear index idx (row of plane z at
-// y) for nx a multiple of 64 and 8-byte aligned fields: the 32 lanes of the warp hold 32
-// consecutive pairs of the row, so the x neighbours outside a pair come from the adjacent
-// lanes; loads and stores are 8-byte vectors. Records hd when hrec is set, writes the mode's
+// y) for even nx and 8-byte aligned fields; loads and stores are 8-byte vectors. LANES (nx a
+// multiple of 64): the 32 lanes of the warp hold 32 consecutive pairs of the row, so the x
+// neighbours outside a pair come from the adjacent lanes; otherwise they are loaded. Records hd when hrec is set, writes the mode's
 // outputs, and returns true with the next stage's m in mn for the RK4 stages.
+template <bool LANES>
 __device__ __forceinline__ bool epilogue_pair(const RowArgs& a, int mode, int z, int y, long long idx, int x0,
                                               int lane, const float (&hd)[2][3], float (&mn)[2][3]) {
   const long long N = a.N;
@@ -195,8 +182,8 @@ __device__ __forceinline__ bool epilogue_pair(const RowArgs& a, int mode, int z,
   const long long oyp = y < ny - 1 ? (long long)nx : ((a.per & 2) ? -wy : 0);
   const long long ozm = z > 0 ? -sz : ((a.per & 4) ? wz : 0);
   const long long ozp = z < a.nz - 1 ? sz : ((a.per & 4) ? -wz : 0);
-  const int oxl = x0 > 0 ? -1 : ((a.per & 1) ? nx - 1 : 0);      // left of x0 (lane 0)
-  const int oxr = x0 + 2 < nx ? 2 : ((a.per & 1) ? 2 - nx : 1);  // right of x0 + 1 (lane 31)
+  const int oxl = x0 > 0 ? -1 : ((a.per & 1) ? nx - 1 : 0);      // left of x0
+  const int oxr = x0 + 2 < nx ? 2 : ((a.per & 1) ? 2 - nx : 1);  // right of x0 + 1
   float mv[2][3], lap[2][3];
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
@@ -209,10 +196,16 @@ __device__ __forceinline__ bool epilogue_pair(const RowArgs& a, int mode, int z,
       zm = *reinterpret_cast<const float2*>(p + ozm);
       zp = *reinterpret_cast<const float2*>(p + ozp);
     }
-    float left = __shfl_up_sync(0xffffffffu, cc.y, 1);
-    float right = __shfl_down_sync(0xffffffffu, cc.x, 1);
-    if (lane == 0) left = p[oxl];
-    if (lane == 31) right = p[oxr];
+    float left, right;
+    if constexpr (LANES) {
+      left = __shfl_up_sync(0xffffffffu, cc.y, 1);
+      right = __shfl_down_sync(0xffffffffu, cc.x, 1);
+      if (lane == 0) left = p[oxl];
+      if (lane == 31) right = p[oxr];
+    } else {
+      left = p[oxl];
+      right = p[oxr];
+    }
     mv[0][c] = cc.x;
     mv[1][c] = cc.y;
     lap[0][c] = a.cx * (left - 2.f * cc.x + cc.y) + a.cy * (ym.x - 2.f * cc.x + yp.x) + a.cz * (zm.x - 2.f * cc.x + zp.x);
@@ -547,9 +540,9 @@ __global__ void __launch_bounds__(3 * RB_ * LX / GBD_E,
       if (stg && !mbar_wait(sbar, 0, GBD_WAIT_LIMIT_NS) && a.status) atomicOr(a.status, GBD_DEV_WAIT_TIMEOUT);
     }
     // 3. epilogue on the real rows: float view of line position x is 2 pad(x/2) + (x & 1).
-    if (KIND == 2 || ((nx % 64) == 0 && a.vec8)) {
-      // Fast path (8-byte aligned fields): an item is a pair of cells (x0, x0 + 1); the 32
-      // lanes of a warp take 32 consecutive pairs of one row (epilogue_pair).
+    if (KIND == 2 || ((nx % 2) == 0 && a.vec8)) {
+      // Fast path (even nx, 8-byte aligned fields): an item is a pair of cells (x0, x0 + 1)
+      // (epilogue_pair).
       const int NP2 = nx / 2;
       bool staged = false;
       if constexpr (SOK) {
@@ -642,7 +635,7 @@ __global__ void __launch_bounds__(3 * RB_ * LX / GBD_E,
         for (int e = threadIdx.x; e < RB * NP2; e += T) {
           const int rr = e / NP2;
           const int xp = e - rr * NP2;
-          if (r0 + rr >= a.rows) continue;  // uniform per warp (NP2 is a multiple of 32)
+          if (r0 + rr >= a.rows) continue;
           int z, y;
           row_zy(rr, z, y);
           const int x0 = 2 * xp;
@@ -668,7 +661,7 @@ __global__ void __launch_bounds__(3 * RB_ * LX / GBD_E,
               hd[1][c] = h2.y * a.hscale;
             }
           }
-          if (epilogue_pair(a, mode, z, y, idx, x0, threadIdx.x & 31, hd, mn) && a.fwd_after) {
+          if (epilogue_pair<false>(a, mode, z, y, idx, x0, 0, hd, mn) && a.fwd_after) {
 #pragma unroll
             for (int c = 0; c < 3; ++c) sm[(c * RB + rr) * LS + pad(xp)] = make_float2(mn[0][c], mn[1][c]);
           }
@@ -851,7 +844,35 @@ static void row_launch_t(const RowArgs* a, const float2* tw, cudaStream_t st) {
   launch_pdl(row_kernel<LX, RB, PREC>, (b.rows + RB - 1) / RB, T, b.stage ? row_stage_smem<LX, RB>() : smem, st, b, tw);
 }
 
-// prec < 0 (with a == nullptr) prepares both precisions
+// Calls f(std::integral_constant<int, RB>) for every tile of length LX until it returns true.
+template <int LX, int PREC, class F>
+static void row_tiles(F f) {
+  constexpr int V0 = row_rb(LX, 0), V1 = row_rb(LX, 1);
+  constexpr int S0 = row_rb_small(LX, PREC, 0), S1 = row_rb_small(LX, PREC, 1), S2 = row_rb_small(LX, PREC, 2);
+  if (f(std::integral_constant<int, V0>())) return;
+  if constexpr (V1 != V0)
+    if (f(std::integral_constant<int, V1>())) return;
+  if constexpr (S0 > 0)
+    if (f(std::integral_constant<int, S0>())) return;
+  if constexpr (S1 > 0)
+    if (f(std::integral_constant<int, S1>())) return;
+  if constexpr (S2 > 0) f(std::integral_constant<int, S2>());
+}
+// Launches (a == nullptr: prepares every tile) length LX with the tile of variant var for a's rows.
+template <int LX, int PREC>
+static void row_launch_tile(int var, const RowArgs* a, const float2* tw, cudaStream_t st) {
+  // (L >= 1024 keeps its four rows: with two, half sectors, 1024x512x1 demag takes 41 us instead of 30)
+  const int rb = a ? pick_tile(a->rows, row_rb(LX, var), LX < 1024 ? row_rb(LX, 0) : 0, row_rb_small(LX, PREC, 2),
+                               row_rb_small(LX, PREC, 1), row_rb_small(LX, PREC, 0))
+                   : 0;
+  row_tiles<LX, PREC>([&](auto r) {
+    constexpr int RB = decltype(r)::value;
+    if (a && rb != RB) return false;
+    row_launch_t<LX, RB, PREC>(a, tw, st);
+    return a != nullptr;
+  });
+}
+
 // Calls f(std::integral_constant<int, LX>) for the x transform length Lx; false for a length
 // without an instantiation.
 template <class F>
@@ -885,11 +906,7 @@ static bool row_switch(int Lx, F f) {
 // parallel.
 template <int PREC>
 bool row_dispatch_p(int Lx, int var, const RowArgs* a, const float2* tw, cudaStream_t st) {
-  return row_switch(Lx, [&](auto lx) {
-    constexpr int LX = decltype(lx)::value;
-    if (var <= 0) row_launch_t<LX, row_rb(LX, 0), PREC>(a, tw, st);
-    if (var != 0) row_launch_t<LX, row_rb(LX, 1), PREC>(a, tw, st);
-  });
+  return row_switch(Lx, [&](auto lx) { row_launch_tile<decltype(lx)::value, PREC>(var, a, tw, st); });
 }
 extern template bool row_dispatch_p<1>(int, int, const RowArgs*, const float2*, cudaStream_t);
 extern template bool row_dispatch_p<2>(int, int, const RowArgs*, const float2*, cudaStream_t);

@@ -19,13 +19,11 @@ bool row_io_dispatch(int Lx, int RB, const RowArgs* a, const float2* tw, cudaStr
   bool done = false;
   row_switch(Lx, [&](auto lx) {
     constexpr int LX = decltype(lx)::value;
-    if (RB == row_rb(LX, 0)) {
-      row_io_launch_t<LX, row_rb(LX, 0)>(a, tw, st);
-      done = true;
-    } else if (RB == row_rb(LX, 1)) {
-      row_io_launch_t<LX, row_rb(LX, 1)>(a, tw, st);
-      done = true;
-    }
+    row_tiles<LX, 0>([&](auto r) {
+      if (RB != decltype(r)::value) return false;
+      row_io_launch_t<LX, decltype(r)::value>(a, tw, st);
+      return done = true;
+    });
   });
   return done;
 }

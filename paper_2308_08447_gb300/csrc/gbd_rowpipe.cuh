@@ -232,7 +232,7 @@ __global__ void __launch_bounds__(3 * pipe_rb(LX) * LX / GBD_E, pipe_blocks(K))
           hd[0][c] = h2.x * a.hscale;
           hd[1][c] = h2.y * a.hscale;
         }
-        if (epilogue_pair(a, mode, z, y0 + rr, idx, 2 * xp, threadIdx.x & 31, hd, mn) && a.fwd_after) {
+        if (epilogue_pair<true>(a, mode, z, y0 + rr, idx, 2 * xp, threadIdx.x & 31, hd, mn) && a.fwd_after) {
 #pragma unroll
           for (int c = 0; c < 3; ++c) lines[(c * RB + rr) * LS + pad(xp)] = make_float2(mn[0][c], mn[1][c]);
         }

@@ -5,20 +5,16 @@
 namespace gbd {
 
 // prec < 0 (with a == nullptr) prepares every precision
-template <int L, int C, bool INV>
-static void ypass_launch_p(int prec, const ColArgs* a, const float2* tw, cudaStream_t st) {
-  if (prec <= 0) ypass_launch_t<L, C, INV, 0>(a, tw, st);
-  if (prec == 1 || prec < 0) ypass_launch_t<L, C, INV, 1>(a, tw, st);
-  if (prec == 2 || prec < 0) ypass_launch_t<L, C, INV, 2>(a, tw, st);
+template <int L, bool INV>
+static bool ypass_launch_p(int var, int prec, const ColArgs* a, const float2* tw, cudaStream_t st) {
+  if (prec <= 0) ypass_launch_tile<L, INV, 0>(var, a, tw, st);
+  if (prec == 1 || prec < 0) ypass_launch_tile<L, INV, 1>(var, a, tw, st);
+  if (prec == 2 || prec < 0) ypass_launch_tile<L, INV, 2>(var, a, tw, st);
+  return true;
 }
 
-#define GBD_Y_CASE(L)                                             \
-  case L:                                                         \
-    if (var <= 0)                                                 \
-      ypass_launch_p<L, ypass_lines(L, 0), INV>(prec, a, tw, st);       \
-    if (var != 0)                                                 \
-      ypass_launch_p<L, ypass_lines(L, 1), INV>(prec, a, tw, st);       \
-    return true;
+#define GBD_Y_CASE(L) \
+  case L: return ypass_launch_p<L, INV>(var, prec, a, tw, st);
 
 template <bool INV>
 static bool ypass_dispatch(int Py, int var, int prec, const ColArgs* a, const float2* tw, cudaStream_t st) {

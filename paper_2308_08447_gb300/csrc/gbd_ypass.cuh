@@ -14,6 +14,7 @@ __global__ void __launch_bounds__(C_ * L / GBD_E, min_blocks(C_ * L / GBD_E))
   constexpr int LS = line_stride<L, false>();
   constexpr int NP = npasses(L, false);
   extern __shared__ float2 sm[];
+  pdl_wait_then_release();
   const long long l0 = (long long)blockIdx.x * LINES;
   const int ny = a.ny;
   const long long nl = a.lines_total;
@@ -62,7 +63,23 @@ static void ypass_launch_t(const ColArgs* a, const float2* tw, cudaStream_t st) 
   constexpr int T = C * L / GBD_E;
   const size_t smem = (size_t)C * line_stride<L, false>() * sizeof(float2);
   prep(y_pass_kernel<L, C, INV, PREC>, smem);
-  if (a) y_pass_kernel<L, C, INV, PREC><<<(unsigned)((a->lines_total + C - 1) / C), T, smem, st>>>(*a, tw);
+  if (a) launch_pdl(y_pass_kernel<L, C, INV, PREC>, (unsigned)((a->lines_total + C - 1) / C), T, smem, st, *a, tw);
+}
+
+// Launches (a == nullptr: prepares every tile of) the y pass of length L with the tile of variant
+// var for a's lines.
+template <int L, bool INV, int PREC>
+static void ypass_launch_tile(int var, const ColArgs* a, const float2* tw, cudaStream_t st) {
+  constexpr int V0 = ypass_lines(L, 0), V1 = ypass_lines(L, 1);
+  constexpr int S0 = ypass_lines_small(L, 0), S1 = ypass_lines_small(L, 1);
+  const int c = a ? pick_tile(a->lines_total, var == 0 ? V0 : V1, V1, S0, S1) : 0;
+  if (!a || c == V0) ypass_launch_t<L, V0, INV, PREC>(a, tw, st);
+  if constexpr (V1 != V0)
+    if (!a || c == V1) ypass_launch_t<L, V1, INV, PREC>(a, tw, st);
+  if constexpr (S0 > 0 && S0 != V1)
+    if (!a || c == S0) ypass_launch_t<L, S0, INV, PREC>(a, tw, st);
+  if constexpr (S1 > 0)
+    if (!a || c == S1) ypass_launch_t<L, S1, INV, PREC>(a, tw, st);
 }
 
 }  // namespace gbd
