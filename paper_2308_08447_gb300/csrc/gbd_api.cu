@@ -360,34 +360,63 @@ static gbd::ColArgs col_args(const gbd_mesh* m) {
   return a;
 }
 
-// Middle of Eq. 1: everything between the forward and the inverse x transforms.
-static void enqueue_conv(gbd_mesh* m, cudaStream_t st) {
+// The whole convolution along y and z in one launch (gbd_small.cu).
+static bool conv_in_one(const gbd::Plan& p) {
+  const bool fp32 = p.film ? gbd::stage_prec(p.prec, p.Py, true) == 0
+                           : gbd::stage_prec(p.prec, p.Py, false) == 0 && gbd::stage_prec(p.prec, p.Pz, true) == 0;
+  return fp32 && gbd::small_conv_ok(p.Hx, p.Py, p.Pz, p.nz, p.per);
+}
+
+// Strides of the z convolution on T [3][nz][Hx][Py], or, when ny = 1, on S [3][nz][Hx].
+static void z_strides(const gbd::Plan& p, gbd::ColArgs& a) {
+  a.Pyq = p.ny > 1 ? p.Py : 1;
+  a.Q = (long long)p.Hx * a.Pyq;
+}
+
+// Middle of Eq. 1: everything between the forward and the inverse x transforms, on the spectra S
+// and T. A 3D convolution that runs in one launch is split into its passes, the same arithmetic,
+// while events time the launches by pass.
+static void enqueue_conv(gbd_mesh* m, float2* S, float2* T, cudaStream_t st) {
   const gbd::Plan& p = m->p;
   gbd::ColArgs a = col_args(m);
+  const bool one = conv_in_one(p);
   if (p.film) {
-    a.dst = m->S;
+    a.dst = S;
     a.Kf = static_cast<const float4*>(m->K);
-    timed(m, GBD_PASS_FILM_CONV, st, [&] { gbd::launch_film_conv(m->p.var_film, m->p.prec, a, m->tw, st); });
+    timed(m, GBD_PASS_FILM_CONV, st, [&] {
+      if (one)
+        gbd::launch_small_conv(a, S, nullptr, 7, m->tw, st);
+      else
+        gbd::launch_film_conv(p.var_film, p.prec, a, m->tw, st);
+    });
     return;
   }
   a.K3 = static_cast<const float2*>(m->K);
+  if (one) {
+    if (m->timing & GBD_TIMING_EVENTS) {
+      timed(m, GBD_PASS_Y_FWD, st, [&] { gbd::launch_small_conv(a, S, T, 1, m->tw, st); });
+      timed(m, GBD_PASS_Z_CONV, st, [&] { gbd::launch_small_conv(a, S, T, 2, m->tw, st); });
+      timed(m, GBD_PASS_Y_INV, st, [&] { gbd::launch_small_conv(a, S, T, 4, m->tw, st); });
+    } else {
+      timed(m, GBD_PASS_Z_CONV, st, [&] { gbd::launch_small_conv(a, S, T, 7, m->tw, st); });
+    }
+    return;
+  }
   if (p.ny > 1) {
     a.lines_total = 3LL * p.nz * p.Hx;
-    a.src = m->S;
-    a.dst = m->T;
-    timed(m, GBD_PASS_Y_FWD, st, [&] { gbd::launch_y_fwd(m->p.var_y, m->p.prec, a, m->tw, st); });
-    a.dst = m->T;
-    a.Q = (long long)p.Hx * p.Py;
-    a.Pyq = p.Py;
-    timed(m, GBD_PASS_Z_CONV, st, [&] { gbd::launch_z_conv(m->p.var_z, m->p.prec, a, m->tw, st); });
-    a.src = m->T;
-    a.dst = m->S;
-    timed(m, GBD_PASS_Y_INV, st, [&] { gbd::launch_y_inv(m->p.var_y, m->p.prec, a, m->tw, st); });
+    a.src = S;
+    a.dst = T;
+    timed(m, GBD_PASS_Y_FWD, st, [&] { gbd::launch_y_fwd(p.var_y, p.prec, a, m->tw, st); });
+    a.dst = T;
+    z_strides(p, a);
+    timed(m, GBD_PASS_Z_CONV, st, [&] { gbd::launch_z_conv(p.var_z, p.prec, a, m->tw, st); });
+    a.src = T;
+    a.dst = S;
+    timed(m, GBD_PASS_Y_INV, st, [&] { gbd::launch_y_inv(p.var_y, p.prec, a, m->tw, st); });
   } else {
-    a.dst = m->S;
-    a.Q = p.Hx;
-    a.Pyq = 1;
-    timed(m, GBD_PASS_Z_CONV, st, [&] { gbd::launch_z_conv(m->p.var_z, m->p.prec, a, m->tw, st); });
+    a.dst = S;
+    z_strides(p, a);
+    timed(m, GBD_PASS_Z_CONV, st, [&] { gbd::launch_z_conv(p.var_z, p.prec, a, m->tw, st); });
   }
 }
 
@@ -534,6 +563,7 @@ gbd_status gbd_mesh_create(const gbd_mesh_desc* desc, gbd_mesh** out) {
   }
   // shared-memory attributes of this mesh's kernels (both tile variants), set now so that
   // later launches, also inside a stream capture, need no configuration call
+  gbd::prepare_small();
   bool have = gbd::prepare_row(p.Lx, p.prec);
   if (p.film) {
     have = have && gbd::prepare_film_conv(p.Py, p.prec);
@@ -778,7 +808,7 @@ gbd_status gbd_demag(gbd_mesh* m, const float* M, float* H, void* stream) {
   a.mode = gbd::ROW_FWD;
   a.fwd_after = 1;
   timed(m, GBD_PASS_ROW_FWD, st, [&] { gbd::launch_row(m->p.Lx, row_var(m, a.mode), m->p.prec, a, m->tw, st); });
-  enqueue_conv(m, st);
+  enqueue_conv(m, m->S, m->T, st);
   a.hscale = 1.f;
   a.out = H;
   a.mode = gbd::ROW_H;
@@ -798,7 +828,7 @@ static gbd_status field_like(gbd_mesh* m, const float* mm, float* out, int mode,
   a.mode = gbd::ROW_FWD;
   a.fwd_after = 1;
   timed(m, GBD_PASS_ROW_FWD, st, [&] { gbd::launch_row(m->p.Lx, row_var(m, a.mode), m->p.prec, a, m->tw, st); });
-  enqueue_conv(m, st);
+  enqueue_conv(m, m->S, m->T, st);
   a.ms = mm;
   a.out = out;
   a.mode = mode;
@@ -893,7 +923,7 @@ static void enqueue_llg_ex(gbd_mesh* m, float* mm, int nsteps, double dt, unsign
           a.hist[k] = m->hist + (size_t)((m->hist_head - k + 5) % 5) * n3;
         }
       } else {
-        enqueue_conv(m, st);
+        enqueue_conv(m, m->S, m->T, st);
       }
       // the next stage needs this stage's forward transform unless it extrapolates
       const bool next_exact = stage == 3 ? !last : !warm;
@@ -1054,7 +1084,7 @@ static void rkf_enqueue_attempt(gbd_mesh* m, const float* mm, double h, const fl
     if (a.extrap) {
       timed(m, GBD_PASS_EXTRAP, st, [&] { gbd::launch_extrap_stage(a, st); });
     } else {
-      enqueue_conv(m, st);
+      enqueue_conv(m, m->S, m->T, st);
       timed(m, GBD_PASS_ROW_RK, st, [&] { gbd::launch_row(m->p.Lx, row_var(m, a.mode), m->p.prec, a, m->tw, st); });
     }
     ms = a.mnext;
@@ -1373,35 +1403,6 @@ constexpr int kNoallocMaxDevices = 64;
 std::mutex g_noalloc_mu;
 void* g_noalloc_addr[kNoallocMaxDevices] = {nullptr};
 
-// Same pass sequence as enqueue_conv, on caller-chosen spectrum buffers.
-void enqueue_conv_on(const gbd_mesh* m, float2* S, float2* T, cudaStream_t st) {
-  const gbd::Plan& p = m->p;
-  gbd::ColArgs a = col_args(m);
-  if (p.film) {
-    a.dst = S;
-    a.Kf = static_cast<const float4*>(m->K);
-    gbd::launch_film_conv(m->p.var_film, m->p.prec, a, m->tw, st);
-    return;
-  }
-  a.K3 = static_cast<const float2*>(m->K);
-  if (p.ny > 1) {
-    a.lines_total = 3LL * p.nz * p.Hx;
-    a.src = S;
-    a.dst = T;
-    gbd::launch_y_fwd(m->p.var_y, m->p.prec, a, m->tw, st);
-    a.Q = (long long)p.Hx * p.Py;
-    a.Pyq = p.Py;
-    gbd::launch_z_conv(m->p.var_z, m->p.prec, a, m->tw, st);
-    a.src = T;
-    a.dst = S;
-    gbd::launch_y_inv(m->p.var_y, m->p.prec, a, m->tw, st);
-  } else {
-    a.dst = S;
-    a.Q = p.Hx;
-    a.Pyq = 1;
-    gbd::launch_z_conv(m->p.var_z, m->p.prec, a, m->tw, st);
-  }
-}
 }  // namespace
 
 extern "C" gbd_status gbd_demag_noalloc(gbd_mesh* m, const float* M, float* H, void* stream) {
@@ -1437,7 +1438,10 @@ extern "C" gbd_status gbd_demag_noalloc(gbd_mesh* m, const float* M, float* H, v
   a.mode = gbd::ROW_FWD;
   a.fwd_after = 1;
   gbd::launch_row(p.Lx, row_var(m, a.mode), p.prec, a, m->tw, st);
-  enqueue_conv_on(m, S, T, st);
+  const int tmp = m->timing;
+  m->timing = 0;   // this call is not traced
+  enqueue_conv(m, S, T, st);
+  m->timing = tmp;
   a.hscale = 1.f;
   a.out = H;
   a.mode = gbd::ROW_H;
@@ -1565,7 +1569,7 @@ cudaError_t time_demag_passes(gbd_mesh* m, cudaStream_t st, float* ms) {
     a.mode = gbd::ROW_FWD;
     a.fwd_after = 1;
     gbd::launch_row(m->p.Lx, row_var(m, a.mode), m->p.prec, a, m->tw, st);
-    enqueue_conv(m, st);
+    enqueue_conv(m, m->S, m->T, st);
     a.out = m->bufB;
     a.mode = gbd::ROW_H;
     a.fwd_after = 0;
@@ -1750,13 +1754,10 @@ extern "C" gbd_status gbd_mesh_autotune(gbd_mesh* m, void* stream) {
         gbd::launch_y_inv(v, p.prec, cb, m->tw, st);
       });
       ca.dst = m->T;
-      ca.Q = (long long)p.Hx * p.Py;
-      ca.Pyq = p.Py;
     } else {
       ca.dst = m->S;
-      ca.Q = p.Hx;
-      ca.Pyq = 1;
     }
+    z_strides(p, ca);
     if (e == cudaSuccess) e = pick(3, [&](int v) { gbd::launch_z_conv(v, p.prec, ca, m->tw, st); });
   }
   if (e != cudaSuccess) return cuda_fail(e, "gbd_mesh_autotune");

@@ -232,6 +232,15 @@ inline int stage_prec(int prec, int L, bool conv) {
       if (radix_at(L, conv, p) == 16) return prec;
   return prec < 0 ? prec : 0;
 }
+// Kernels for meshes that do not fill the GPU (FP32; gbd_small.cu), whatever the tile variant.
+bool small_row_ok(int Lx, int rows);
+bool launch_small_row(int Lx, const RowArgs& a, const float2* tw, cudaStream_t st);
+// The convolution between the x passes, S [3][nz][Hx][ny] in place, one block per kx. phases: 7, or
+// 1 (y FFT, S to T), 2 (z FFT, product, z IFFT on T), 4 (y IFFT, T to S) as launches of their own.
+bool small_conv_ok(int Hx, int Py, int Pz, int nz, int per);
+bool launch_small_conv(const ColArgs& a, float2* S, float2* T, int phases, const float2* tw, cudaStream_t st);
+void prepare_small();
+
 // Set the kernels' shared-memory attribute for both variants of a length without launching
 // (done when a mesh is created, so later launches inside a stream capture need no driver
 // configuration call). Return false for a length without an instantiation.

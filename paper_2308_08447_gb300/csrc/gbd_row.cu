@@ -128,6 +128,8 @@ static void set_vec8(RowArgs& a) {
 bool launch_row(int Lx, int var, int prec, const RowArgs& a0, const float2* tw, cudaStream_t st) {
   RowArgs a = a0;
   set_vec8(a);
+  prec = stage_prec(prec, Lx, false);
+  if (prec == 0 && small_row_ok(Lx, a.rows)) return launch_small_row(Lx, a, tw, st);
   if (mixed_len(Lx)) return prec == 0 && row_dispatch_mixed(Lx, var, &a, tw, st);
   if (var >= 2 && prec == 0) {
     const int kind = pipe_kind(Lx, a, var);
@@ -214,6 +216,7 @@ void launch_extrap_stage(const RowArgs& a0, cudaStream_t st) {
   launch_pdl(extrap_stage_kernel, (unsigned)((items + 255) / 256), 256, 0, st, a);
 }
 bool prepare_row(int Lx, int prec) {
+  prec = stage_prec(prec, Lx, false);
   if (mixed_len(Lx)) return prec <= 0 && row_dispatch_mixed(Lx, -1, nullptr, nullptr, nullptr);
   if (prec <= 0) pipe_dispatch(Lx, -1, nullptr, nullptr, nullptr);
   return row_dispatch(Lx, -1, prec, nullptr, nullptr, nullptr);
