@@ -122,6 +122,26 @@ static void set_vec8(RowArgs& a) {
   a.vec8 = ok ? 1 : 0;
 }
 
+static bool transform_only(const RowArgs& a) { return a.mode == ROW_FWD || (a.mode == ROW_H && !a.extrap); }
+
+// Whether an FP32 launch takes the paired kernel (gbd_rowpair.cuh), whatever the tile variant. It needs
+// an open x. Both sides measured (whole demag or RK stage of the mesh, us, row_kernel / paired):
+//   - lengths 3 * 2^k, 5 * 2^k: always (320x320x4 72 / 61, 1200x600x1 demag 76 / 64; 384x384x64 forward
+//     rows 261 / 132);
+//   - L >= 1024 (one pair per block: half sectors of the spectrum): only stages that row_kernel's staged
+//     instances do not serve (800x800x1 63 / 57; with them 1024x1024x1 61.5 / 67, 1024x512x2 106 / 114);
+//   - below, transforms: 3D meshes and films of 1024 rows (256x256x8 58 / 54, 512x512x64 forward rows 204
+//     / 193, 512x1024x1 43 / 39; shorter films 512x512x1 21 / 23);
+//   - below, epilogues: 3D meshes and films that give 90 blocks (480x240x2 39 / 34, 512x512x1 30 / 27,
+//     400x400x1 30 / 26; 256x512x1 15 / 17).
+static bool take_pair(int Lx, const RowArgs& a) {
+  if (mixed_len(Lx)) return true;
+  if ((a.per & 1) || Lx < 32) return false;
+  if (Lx >= 1024) return !transform_only(a) && (a.nx % 64 != 0 || a.ny % 4 != 0);
+  if (transform_only(a)) return a.nz > 1 || a.rows >= 1024;
+  return a.nz > 1 || a.rows >= 90 * 2 * (1024 / Lx);
+}
+
 // Tile variants 2 and 3 are the persistent pipelined kernel (gbd_rowpipe.cuh, FP32 only) where it
 // applies (3: the RK stages stage only the spectrum tile, two blocks per SM); other launches of
 // variants 2 and 3 take row_kernel's variant 1.
@@ -130,7 +150,9 @@ bool launch_row(int Lx, int var, int prec, const RowArgs& a0, const float2* tw, 
   set_vec8(a);
   prec = stage_prec(prec, Lx, false);
   if (prec == 0 && small_row_ok(Lx, a.rows)) return launch_small_row(Lx, a, tw, st);
-  if (mixed_len(Lx)) return prec == 0 && row_dispatch_mixed(Lx, var, &a, tw, st);
+  if (prec == 0 && take_pair(Lx, a))
+    return transform_only(a) ? pair_dispatch_io(Lx, &a, tw, st)
+                             : pair_dispatch_epi(Lx, &a, tw, st) || pair_dispatch_epi_mixed(Lx, &a, tw, st);
   if (var >= 2 && prec == 0) {
     const int kind = pipe_kind(Lx, a, var);
     if (kind >= 0) return pipe_dispatch(Lx, kind, &a, tw, st);
@@ -217,7 +239,11 @@ void launch_extrap_stage(const RowArgs& a0, cudaStream_t st) {
 }
 bool prepare_row(int Lx, int prec) {
   prec = stage_prec(prec, Lx, false);
-  if (mixed_len(Lx)) return prec <= 0 && row_dispatch_mixed(Lx, -1, nullptr, nullptr, nullptr);
+  if (prec <= 0) {
+    pair_dispatch_io(Lx, nullptr, nullptr, nullptr);
+    pair_dispatch_epi(Lx, nullptr, nullptr, nullptr);
+  }
+  if (mixed_len(Lx)) return prec <= 0 && pair_dispatch_epi_mixed(Lx, nullptr, nullptr, nullptr);
   if (prec <= 0) pipe_dispatch(Lx, -1, nullptr, nullptr, nullptr);
   return row_dispatch(Lx, -1, prec, nullptr, nullptr, nullptr);
 }
