@@ -217,10 +217,13 @@ bool row_io_dispatch(int Lx, int RB, const RowArgs* a, const float2* tw, cudaStr
 // The staged RK-stage instances (row kernel KIND 2, FP32, power-of-two Lx; gbd_row_rk.cu), likewise.
 bool row_rk_dispatch(int Lx, int RB, const RowArgs* a, const float2* tw, cudaStream_t st);
 
-// The paired x-row kernels (FP32, open x; gbd_rowpair.cuh): the launches with an epilogue, and the
-// transform-only ones; false for a length without an instance. a == nullptr prepares.
+// The paired x-row kernels (FP32, open x; gbd_rowpair.cuh): the launches with an epilogue (RK4 stages
+// and the others), and the transform-only ones; false for a length without an instance. a == nullptr
+// prepares.
 bool pair_dispatch_epi(int Lx, const RowArgs* a, const float2* tw, cudaStream_t st);
-bool pair_dispatch_epi_mixed(int Lx, const RowArgs* a, const float2* tw, cudaStream_t st);
+bool pair_dispatch_rk(int Lx, const RowArgs* a, const float2* tw, cudaStream_t st);
+bool pair_dispatch_rk_mixed(int Lx, const RowArgs* a, const float2* tw, cudaStream_t st);
+bool pair_dispatch_other(int Lx, const RowArgs* a, const float2* tw, cudaStream_t st);
 bool pair_dispatch_io(int Lx, const RowArgs* a, const float2* tw, cudaStream_t st);
 
 // Transform lengths 3 * 2^k and 5 * 2^k (FP32 only; gbd_mixed_conv.cu): the launchers above forward

@@ -151,8 +151,7 @@ bool launch_row(int Lx, int var, int prec, const RowArgs& a0, const float2* tw, 
   prec = stage_prec(prec, Lx, false);
   if (prec == 0 && small_row_ok(Lx, a.rows)) return launch_small_row(Lx, a, tw, st);
   if (prec == 0 && take_pair(Lx, a))
-    return transform_only(a) ? pair_dispatch_io(Lx, &a, tw, st)
-                             : pair_dispatch_epi(Lx, &a, tw, st) || pair_dispatch_epi_mixed(Lx, &a, tw, st);
+    return transform_only(a) ? pair_dispatch_io(Lx, &a, tw, st) : pair_dispatch_epi(Lx, &a, tw, st);
   if (var >= 2 && prec == 0) {
     const int kind = pipe_kind(Lx, a, var);
     if (kind >= 0) return pipe_dispatch(Lx, kind, &a, tw, st);
@@ -243,7 +242,7 @@ bool prepare_row(int Lx, int prec) {
     pair_dispatch_io(Lx, nullptr, nullptr, nullptr);
     pair_dispatch_epi(Lx, nullptr, nullptr, nullptr);
   }
-  if (mixed_len(Lx)) return prec <= 0 && pair_dispatch_epi_mixed(Lx, nullptr, nullptr, nullptr);
+  if (mixed_len(Lx)) return prec <= 0 && pair_dispatch_epi(Lx, nullptr, nullptr, nullptr);
   if (prec <= 0) pipe_dispatch(Lx, -1, nullptr, nullptr, nullptr);
   return row_dispatch(Lx, -1, prec, nullptr, nullptr, nullptr);
 }

@@ -19,7 +19,7 @@ __host__ __device__ constexpr int pair_threads(int L, int npr) { return 3 * npr 
 // the film's stage takes 62 us instead of 47), the transform-only ones at 18 (96 registers; 512x512x64
 // forward 238 us at 16 warps, 194 at 18).
 __host__ __device__ constexpr int pair_blocks(int T, int kind) {
-  const int warps = kind == 0 ? 16 : 18, w = (T + 31) / 32;
+  const int warps = kind != 1 ? 16 : 18, w = (T + 31) / 32;
   return warps / w < 1 ? 1 : warps / w;
 }
 template <int L, int NPR>
@@ -27,10 +27,13 @@ __host__ __device__ constexpr size_t pair_smem() {
   return (size_t)3 * NPR * line_stride<L, true>() * sizeof(cpair);
 }
 
-// The RK4 stages of the cells (x0, x0 + 1) of the rows y, y + 1 of plane z (linear index idx of the
-// first), with the demag field in hd and the next stage's m out in mn, [row][cell][component]: all
-// loads first, then epilogue_pair's arithmetic, term for term. even nx, 8-byte aligned fields.
-__device__ __forceinline__ void epilogue_rows2(const RowArgs& a, int mode, int z, int y, long long idx, int x0,
+// The epilogue of the cells (x0, x0 + 1) of the rows y, y + 1 of plane z (linear index idx of the
+// first), with the demag field in hd, for every mode but ROW_H: all loads first, then epilogue_pair's
+// arithmetic, term for term. Returns true with the next stage's m in mn ([row][cell][component]) for
+// the RK stages that have one. Even nx, 8-byte aligned fields, open x. RK4: the modes ROW_RK1 .. 4, or
+// the others (one function for both costs the RK4 stages registers).
+template <bool RK4>
+__device__ __forceinline__ bool epilogue_rows2(const RowArgs& a, int mode, int z, int y, long long idx, int x0,
                                                const float (&hd)[2][2][3], float (&mn)[2][2][3]) {
   const long long N = a.N;
   const int nx = a.nx, ny = a.ny;
@@ -41,27 +44,29 @@ __device__ __forceinline__ void epilogue_rows2(const RowArgs& a, int mode, int z
   const long long ozm = z > 0 ? -sz : ((a.per & 4) ? wz : 0);
   const long long ozp = z < a.nz - 1 ? sz : ((a.per & 4) ? -wz : 0);
   const int oxl = x0 > 0 ? -1 : 0, oxr = x0 + 2 < nx ? 2 : 1;   // free x boundary
-  const bool rk_acc = mode != ROW_RK1;
+  const bool rk_acc = RK4 && mode != ROW_RK1;
+  const bool rkg = !RK4 && mode == ROW_RKG;
   float mv[2][2][3], lap[2][2][3];
-  float2 q0[2][3], qa[2][3];
+  float2 q0[2][3], qa[2][3];   // step-start m; k-sum, or (ROW_RKG) the weighted sum of earlier slopes
+  auto ld2 = [](const float* p) { return *reinterpret_cast<const float2*>(p); };
+  auto st2 = [](float* p, float x, float y) { *reinterpret_cast<float2*>(p) = make_float2(x, y); };
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     const float* __restrict__ p = a.ms + c * N + idx;
-    auto at = [&](long long o) { return *reinterpret_cast<const float2*>(p + o); };
-    const float2 r[4] = {at(oym), at(0), at(nx), at(oyp)};
+    const float2 r[4] = {ld2(p + oym), ld2(p), ld2(p + nx), ld2(p + oyp)};
     const float left[2] = {p[oxl], p[nx + oxl]}, right[2] = {p[oxr], p[nx + oxr]};
     float2 zm[2] = {r[1], r[2]}, zp[2] = {r[1], r[2]};
     if (a.nz > 1) {
-      zm[0] = at(ozm);
-      zm[1] = at(ozm + nx);
-      zp[0] = at(ozp);
-      zp[1] = at(ozp + nx);
+      zm[0] = ld2(p + ozm);
+      zm[1] = ld2(p + ozm + nx);
+      zp[0] = ld2(p + ozp);
+      zp[1] = ld2(p + ozp + nx);
     }
     if (rk_acc) {
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
-        q0[u][c] = *reinterpret_cast<const float2*>(a.m0 + c * N + idx + u * nx);
-        qa[u][c] = *reinterpret_cast<const float2*>(a.acc + c * N + idx + u * nx);
+        q0[u][c] = ld2(a.m0 + c * N + idx + u * nx);
+        qa[u][c] = ld2(a.acc + c * N + idx + u * nx);
       }
     }
 #pragma unroll
@@ -75,12 +80,34 @@ __device__ __forceinline__ void epilogue_rows2(const RowArgs& a, int mode, int z
                      a.cz * (zm[u].y - 2.f * cc.y + zp[u].y);
     }
   }
+  const float hs = rkg && a.hdev ? *a.hdev : 1.f;   // step size on the device, or folded into kw
+  if (rkg && a.mnext) {
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) q0[u][c] = ld2(a.m0 + c * N + idx + u * nx);
+    for (int j = 0; j < a.nk; ++j) {
+      const float* kj = a.kin[j] + idx;
+      const float w = a.kw[j] * hs;
+      float2 k[2][3];
+#pragma unroll
+      for (int u = 0; u < 2; ++u)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) k[u][c] = ld2(kj + c * N + u * nx);
+#pragma unroll
+      for (int u = 0; u < 2; ++u)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          q0[u][c].x = fmaf(w, k[u][c].x, q0[u][c].x);
+          q0[u][c].y = fmaf(w, k[u][c].y, q0[u][c].y);
+        }
+    }
+  }
   if (a.hrec) {
 #pragma unroll
     for (int u = 0; u < 2; ++u)
 #pragma unroll
-      for (int c = 0; c < 3; ++c)
-        *reinterpret_cast<float2*>(a.hrec + c * N + idx + u * nx) = make_float2(hd[u][0][c], hd[u][1][c]);
+      for (int c = 0; c < 3; ++c) st2(a.hrec + c * N + idx + u * nx, hd[u][0][c], hd[u][1][c]);
   }
 #pragma unroll
   for (int u = 0; u < 2; ++u) {
@@ -94,24 +121,37 @@ __device__ __forceinline__ void epilogue_rows2(const RowArgs& a, int mode, int z
         accv[1][c] = qa[u][c].y;
       }
     }
+    const int lm = rkg ? (int)ROW_RHS : mode;
 #pragma unroll
     for (int v = 0; v < 2; ++v)
-      llg_update(a, mode, hd[u][v], mv[u][v], lap[u][v], m0v[v], accv[v], mn[u][v], ao[v], res[v]);
+      llg_update(a, lm, hd[u][v], mv[u][v], lap[u][v], m0v[v], accv[v], mn[u][v], ao[v], res[v]);
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      const float2 v = make_float2(mn[u][0][c], mn[u][1][c]);
-      if (mode == ROW_RK4) {   // m0_out may alias m0: each cell is read, then written, by one thread
-        *reinterpret_cast<float2*>(a.m0_out + c * N + idx + u * nx) = v;
+      const long long o = c * N + idx + u * nx;
+      if (!RK4 && !rkg) {
+        st2(a.out + o, res[0][c], res[1][c]);
+      } else if (rkg) {
+        st2(a.kout + o, res[0][c], res[1][c]);
+        if (a.mnext) {
+          const float w = a.kw[a.nk] * hs;
+          mn[u][0][c] = fmaf(w, res[0][c], q0[u][c].x);
+          mn[u][1][c] = fmaf(w, res[1][c], q0[u][c].y);
+          st2(a.mnext + o, mn[u][0][c], mn[u][1][c]);
+        }
+      } else if (mode == ROW_RK4) {   // m0_out may alias m0: each cell is read, then written, by one thread
+        st2(a.m0_out + o, mn[u][0][c], mn[u][1][c]);
       } else {
-        *reinterpret_cast<float2*>(a.acc + c * N + idx + u * nx) = make_float2(ao[0][c], ao[1][c]);
-        *reinterpret_cast<float2*>(a.mnext + c * N + idx + u * nx) = v;
+        st2(a.acc + o, ao[0][c], ao[1][c]);
+        st2(a.mnext + o, mn[u][0][c], mn[u][1][c]);
       }
     }
   }
+  return RK4 || (rkg && a.mnext);
 }
 
-// KIND 0: every mode with an epilogue; KIND 1: the forward transform, and the inverse transform to
-// hscale * H_d.
+// KIND 0: the RK4 stages; KIND 1: the forward transform, and the inverse transform to hscale * H_d;
+// KIND 2: the other epilogues (H_eff, dm/dt, general RK stages; in one instance with the RK4 stages
+// their code costs those 3 %).
 template <int L, int NPR, int KIND>
 __global__ void __launch_bounds__(pair_threads(L, NPR), pair_blocks(pair_threads(L, NPR), KIND))
     row_pair_kernel(const __grid_constant__ RowArgs a, const float2* __restrict__ tw) {
@@ -126,6 +166,8 @@ __global__ void __launch_bounds__(pair_threads(L, NPR), pair_blocks(pair_threads
   const long long N = a.N;
   const int mode = a.mode, nx = a.nx, ny = a.ny;
   const int tid = threadIdx.x;
+  if constexpr (KIND == 0) __builtin_assume(mode >= ROW_RK1 && mode <= ROW_RK4);
+  if constexpr (KIND == 2) __builtin_assume(mode == ROW_HEFF || mode == ROW_RHS || mode == ROW_RKG);
   // transform items: pair line (g, c) and positions jj + i L/16
   const int tg = tid % NPR, tt = tid / NPR, jj = tt % LT, tc = tt / LT;
   cpair* const tl = smp + (tc * NPR + tg) * LS;
@@ -172,7 +214,7 @@ __global__ void __launch_bounds__(pair_threads(L, NPR), pair_blocks(pair_threads
   const long long kstep = (long long)LT * ny;
   pdl_wait_then_release();
 
-  if (mode != ROW_FWD) {
+  if (KIND != 1 || mode != ROW_FWD) {
     if (KIND == 1 || !a.extrap) {
       // 1. X[k], X[L - k] -> Z[k], Z[L - k], k = jj + i L/16 < L/2 (k = 0 with X[L], and X[L/2] alone):
       //    every thread issues all its loads before using any
@@ -256,7 +298,6 @@ __global__ void __launch_bounds__(pair_threads(L, NPR), pair_blocks(pair_threads
       };
       if ((nx & 1) == 0 && a.vec8) {
         const int NP2 = nx / 2;
-        const bool rk = mode >= ROW_RK1 && mode <= ROW_RK4;
         for (int e = tid; e < NPR * NP2; e += T) {
           const int g = NPR == 1 ? 0 : e / NP2, p = e - g * NP2;
           const int row = r0 + 2 * g;
@@ -266,8 +307,8 @@ __global__ void __launch_bounds__(pair_threads(L, NPR), pair_blocks(pair_threads
           float hd[2][2][3], mn[2][2][3] = {};
           if (!a.extrap) field(g, p, hd);
           bool next = a.fwd_after != 0;
-          if (rk && !a.extrap && y + 1 < ny) {
-            epilogue_rows2(a, mode, z, y, idx, 2 * p, hd, mn);
+          if (!a.extrap && y + 1 < ny) {
+            next = epilogue_rows2<KIND == 0>(a, mode, z, y, idx, 2 * p, hd, mn) && next;
           } else {
 #pragma unroll 1
             for (int u = 0; u < 2; ++u) {
@@ -366,7 +407,7 @@ __global__ void __launch_bounds__(pair_threads(L, NPR), pair_blocks(pair_threads
   }
   // 4. zero what the forward transform reads beyond the data (cells nx .. L - 1; rows past the last)
   {
-    const int p0 = (mode == ROW_FWD) ? (nx + 1) / 2 : nx / 2;   // first element with a zero cell
+    const int p0 = KIND == 1 ? (nx + 1) / 2 : nx / 2;   // first element with a zero cell
     for (int line = 0; line < LINES; ++line) {
       float4* fl = reinterpret_cast<float4*>(smp + line * LS);
       for (int p = p0 + tid; p < HALF; p += T) {
@@ -378,7 +419,7 @@ __global__ void __launch_bounds__(pair_threads(L, NPR), pair_blocks(pair_threads
         }
       }
     }
-    if (KIND == 0 && r0 + 2 * NPR > a.rows && mode != ROW_FWD) {
+    if (KIND != 1 && r0 + 2 * NPR > a.rows) {
       for (int rr = 0; rr < 2 * NPR; ++rr)
         if (r0 + rr >= a.rows)
           for (int c = 0; c < 3; ++c)

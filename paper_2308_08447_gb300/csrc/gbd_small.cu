@@ -72,6 +72,8 @@ __device__ __forceinline__ void load_twiddles(const FftPlan& f, float2* stw, con
   }
 }
 
+__device__ __forceinline__ void prefetch_l1(const void* p) { asm volatile("prefetch.global.L1 [%0];\n" ::"l"(p)); }
+
 // One radix-R butterfly: twiddles from the shared table (sign S), DFT.
 template <int S, int R>
 __device__ __forceinline__ void small_butterfly(float2* v, const float2* __restrict__ t, int k, int ns) {
@@ -230,12 +232,13 @@ __global__ void __launch_bounds__(384, 2) small_row_kernel(const __grid_constant
 
   if (mode != ROW_FWD && !a.extrap) {
     // 1. X[k], X[L - k] (global, [kx][y] layout) -> Z in the lines; all loads of a thread first
-    constexpr int IPT = 5;   // 3 RB (L/2 + 1) items over at least 3 RB L / 8 threads (fewer: more rounds)
-    const int items = lines * (HALF + 1);
+    constexpr int IPT = 5;   // covers T >= 3 RB L / 8; a block with more threads runs fewer
+    const int items = lines * (HALF + 1), rounds = (items + T - 1) / T;
     for (int e0 = tid; e0 < items; e0 += IPT * T) {
       float2 A[IPT], B[IPT];
 #pragma unroll
       for (int i = 0; i < IPT; ++i) {
+        if (i >= rounds) break;
         const int e = e0 + i * T;
         A[i] = B[i] = make_float2(0.f, 0.f);
         if (e < items) {
@@ -252,6 +255,7 @@ __global__ void __launch_bounds__(384, 2) small_row_kernel(const __grid_constant
       }
 #pragma unroll
       for (int i = 0; i < IPT; ++i) {
+        if (i >= rounds) break;
         const int e = e0 + i * T;
         if (e < items) {
           const int rr = e & (RB - 1), t2 = e >> s.rb_log;
@@ -511,6 +515,9 @@ __global__ void __launch_bounds__(384, PZ >= 16 ? 1 : 2) small_conv_kernel(const
   float2* Y = X + lines * f.ls;
   float2* stw = Y + lines * f.ls;
   if (s.phases & 5) load_twiddles(f, stw, tw);
+  // a film's kernel entry of the thread's first column towards L1, ahead of the wait (with layers, the
+  // dozen entries per thread displace more than they save: 480x240x2 stage 33.6 -> 34.5 us)
+  if (PZ == 1 && tid < L) prefetch_l1(a.Kf + (long long)kx * KY + (tid > L / 2 ? L - tid : tid));
   pdl_wait_then_release();
   __syncthreads();
   auto gS = [&](int l) { return s.S + ((long long)l * a.Hx + kx) * ny; };
@@ -599,7 +606,12 @@ __global__ void __launch_bounds__(384, PZ >= 16 ? 1 : 2) small_conv_kernel(const
 constexpr size_t kSmallSmem = 232448;   // dynamic shared memory of a block
 constexpr int kSmallThreads = 384;
 
-static int small_threads(int values) { return std::min(kSmallThreads, (values / 8 + 31) / 32 * 32); }
+// Threads of a block: one per x-row item or y frequency while the blocks leave SMs to spare (96x64x1
+// stage 10.4 -> 9.1 us), else one per eight values (the eight-mesh batch 6620 -> 6370 us).
+static int small_threads(int blocks, int items, int values) {
+  const int t = blocks <= 2 * kTileBlocks ? items : values / 8;
+  return std::min(kSmallThreads, (t + 31) / 32 * 32);
+}
 
 static size_t small_row_smem(const FftPlan& f, int RB, int nx, int stage_rows) {
   return (size_t)((2 * 3 * RB * f.ls + f.ntw + f.L / 2 + 2) & ~1) * sizeof(float2) + (size_t)stage_rows * 3 * nx * 4 + 16;
@@ -648,7 +660,8 @@ bool launch_small_row(int Lx, const RowArgs& a, const float2* tw, cudaStream_t s
     if (a.nz > 1 && smem_of(s.staged | 2) <= kSmallSmem / 2) s.staged |= 2;
   }
   const size_t smem = smem_of(s.staged);
-  launch_pdl(small_row_kernel, (unsigned)((a.rows + RB - 1) >> s.rb_log), (unsigned)small_threads(3 * RB * Lx), smem, st, s, tw);
+  const int blocks = (a.rows + RB - 1) >> s.rb_log;
+  launch_pdl(small_row_kernel, (unsigned)blocks, (unsigned)small_threads(blocks, 3 * RB * (Lx / 2 + 1), 3 * RB * Lx), smem, st, s, tw);
   return true;
 }
 
@@ -674,7 +687,8 @@ bool launch_small_conv(const ColArgs& a, float2* S, float2* T, int phases, const
   s.phases = phases;
   if (!make_fft_plan(a.Py, s.f)) return false;
   const size_t smem = small_conv_smem(s.f, a.nz);
-  const unsigned threads = (unsigned)small_threads(3 * a.nz * a.Py);
+  const int values = 3 * a.nz * a.Py;
+  const unsigned threads = (unsigned)small_threads(a.Hx, std::max(a.Py, values / 8), values);
   switch (a.Pz) {
     case 1: launch_pdl(small_conv_kernel<1>, a.Hx, threads, smem, st, s, tw); return true;
     case 4: launch_pdl(small_conv_kernel<4>, a.Hx, threads, smem, st, s, tw); return true;
