@@ -311,6 +311,27 @@ static void mark_done(gbd_mesh* m, cudaStream_t st) {
   m->done.emplace_back(st, ev);
 }
 
+// Twiddle levels: exp(-2 pi i m / N) at index tw_base(N) + m for m < N and N = 1, 2, 4, ...,
+// GBD_TW_LEN, N = 3, 6, ..., GBD_TW3_MAX and N = 5, 10, ..., GBD_TW5_MAX, FP64 on the host, rounded
+// to FP32 (the split DFT-16 fragment tables between them are written on the device). The same for
+// every mesh: computed once per process (80,000 sines and cosines, most of a mesh's creation time).
+static const std::vector<float2>& twiddle_levels() {
+  static const std::vector<float2> table = [] {
+    std::vector<float2> tw(GBD_TW_TOTAL, make_float2(1.f, 0.f));
+    auto level = [&](int N) {
+      for (int k = 0; k < N; ++k) {
+        const double ang = -2.0 * 3.14159265358979323846264338327950288 * (double)k / N;
+        tw[gbd::tw_base(N) + k] = make_float2((float)std::cos(ang), (float)std::sin(ang));
+      }
+    };
+    for (int N = 1; N <= GBD_TW_LEN; N *= 2) level(N);
+    for (int N = 3; N <= GBD_TW3_MAX; N *= 2) level(N);
+    for (int N = 5; N <= GBD_TW5_MAX; N *= 2) level(N);
+    return tw;
+  }();
+  return table;
+}
+
 // ---- launch sequences ------------------------------------------------------------------------
 
 // Tile variant of an x-row launch: the transform-only launches (forward, or inverse to H_d) and
@@ -529,20 +550,7 @@ gbd_status gbd_mesh_create(const gbd_mesh_desc* desc, gbd_mesh** out) {
                   std::string("cudaMallocAsync: ") + cudaGetErrorString(e));
     }
   }
-  // twiddle levels: exp(-2 pi i m / N) at index tw_base(N) + m for m < N and N = 1, 2, 4, ...,
-  // GBD_TW_LEN, N = 3, 6, ..., GBD_TW3_MAX and N = 5, 10, ..., GBD_TW5_MAX, FP64 on the host,
-  // rounded to FP32 (the split DFT-16 fragment tables between them are written on the device
-  // below)
-  std::vector<float2> tw(GBD_TW_TOTAL, make_float2(1.f, 0.f));
-  auto level = [&](int N) {
-    for (int k = 0; k < N; ++k) {
-      const double ang = -2.0 * 3.14159265358979323846264338327950288 * (double)k / N;
-      tw[gbd::tw_base(N) + k] = make_float2((float)std::cos(ang), (float)std::sin(ang));
-    }
-  };
-  for (int N = 1; N <= GBD_TW_LEN; N *= 2) level(N);
-  for (int N = 3; N <= GBD_TW3_MAX; N *= 2) level(N);
-  for (int N = 5; N <= GBD_TW5_MAX; N *= 2) level(N);
+  const std::vector<float2>& tw = twiddle_levels();
   cudaStream_t ls = lib_stream(m->device);
   m->status = reinterpret_cast<unsigned*>(m->tw + GBD_TW_TOTAL);
   // test hook: GBD_TEST_WAIT_TIMEOUT=1 makes this mesh's staged RK-stage copies expect 16 bytes
