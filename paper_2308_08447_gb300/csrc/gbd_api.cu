@@ -922,14 +922,27 @@ static void enqueue_llg_ex(gbd_mesh* m, float* mm, int nsteps, double dt, unsign
         a.hrec = m->hist + (size_t)m->hist_head * n3;
         if (m->hist_count < 5) ++m->hist_count;
       }
-      if (warm && stage > 0) {
+      a.hx0 = a.hx1 = nullptr;
+      if (warm && stage == 1) {
+        // stage 2 reads the five fields once for all three stages: it keeps its own, at t + dt/2, for
+        // stage 3 in the x spectrum's buffer, free until stage 4's forward transform (at least 12 bytes
+        // per cell), and stage 4's, at t + dt, in place of the oldest field, which the next step's first
+        // stage replaces
         a.extrap = 1;
         a.nh = 5;
-        const float* w = (stage == 3) ? w_one : w_half;
         for (int k = 0; k < 5; ++k) {
-          a.hw[k] = w[k];
+          a.hw[k] = w_half[k];
+          a.hw1[k] = w_one[k];
           a.hist[k] = m->hist + (size_t)((m->hist_head - k + 5) % 5) * n3;
         }
+        a.hx0 = reinterpret_cast<float*>(m->S);
+        a.hx1 = m->hist + (size_t)((m->hist_head + 1) % 5) * n3;
+      } else if (warm && stage > 1) {
+        a.extrap = 1;
+        a.nh = 1;
+        a.hw[0] = 1.f;
+        a.hist[0] = stage == 2 ? reinterpret_cast<const float*>(m->S) : m->hist + (size_t)((m->hist_head + 1) % 5) * n3;
+        for (int k = 1; k < 5; ++k) a.hist[k] = nullptr;
       } else {
         enqueue_conv(m, m->S, m->T, st);
       }

@@ -132,10 +132,14 @@ struct RowArgs {
   // sum_{k < nh} hw[k] hist[k] over the step-start history (newest first) and no inverse transform
   // runs; hrec, when set, receives the stage's demag field (hscale * H_d), [3][N]
   int extrap;
-  int nh;                   // history terms used (5 for RK4, 6 for RKF5(6))
+  int nh;                   // history terms used (5 for RK4, 6 for RKF5(6), 1: the field itself)
   float hw[6];
   const float* hist[6];
   float* hrec;
+  // with nh = 5 and hx0 set, the stage also keeps its own field in hx0 (the next stage's, at the same
+  // time) and the combination with the weights hw1 in hx1 (the stage after that); hx1 may be hist[4]
+  float *hx0, *hx1;
+  float hw1[5];
   // general explicit RK stage (ROW_RKG): kin[0..nk) are earlier stages' dm/dt, kw their
   // weights dt a_(i+1),j, kw[nk] the weight of this stage's k; mnext may be null (last stage).
   // With hdev set the step size lives on the device: kw holds a_(i+1),j and is scaled by *hdev.

@@ -71,7 +71,7 @@ __global__ void __launch_bounds__(256) rkf_final_kernel(const RkfArgs a) {
 // Extrapolated RK4 stage without a transform (stages 2 and 3, and a last stage 4): the
 // epilogue alone over all cells, the demag field from the history. One thread per pair of
 // cells (nx % 64 == 0, 8-byte aligned fields) or per cell.
-__global__ void __launch_bounds__(256) extrap_stage_kernel(const RowArgs a) {
+__global__ void __launch_bounds__(256) extrap_stage_kernel(const __grid_constant__ RowArgs a) {
   pdl_wait_then_release();
   const int nx = a.nx, ny = a.ny;
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;

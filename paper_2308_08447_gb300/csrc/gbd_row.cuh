@@ -112,47 +112,79 @@ __device__ __forceinline__ void llg_update(const RowArgs& a, int mode, const flo
 }
 
 // Extrapolated demag field (sum_k hw[k] hist[k], k < NH) of cells idx, idx + 1. NH is a
-// template argument so that all history loads of a thread issue back to back.
-template <int NH>
+// template argument so that all history loads of a thread issue back to back. KEEP: also store it,
+// and the combination with the weights hw1 (RowArgs::hx0, hx1; all of a cell's history is read before
+// its hx1 is written).
+template <int NH, bool KEEP>
 __device__ __forceinline__ void extrap_pair_n(const RowArgs& a, long long idx, float (&hd)[2][3]) {
+  float2 v[3][NH];
+#pragma unroll
+  for (int c = 0; c < 3; ++c)
+#pragma unroll
+    for (int k = 0; k < NH; ++k) v[c][k] = *reinterpret_cast<const float2*>(a.hist[k] + c * a.N + idx);
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    float2 h2 = make_float2(0.f, 0.f);
+    float2 h2 = make_float2(0.f, 0.f), g2 = make_float2(0.f, 0.f);
 #pragma unroll
     for (int k = 0; k < NH; ++k) {
-      const float2 hk = *reinterpret_cast<const float2*>(a.hist[k] + c * a.N + idx);
+      const float2 hk = v[c][k];
       h2.x = fmaf(a.hw[k], hk.x, h2.x);
       h2.y = fmaf(a.hw[k], hk.y, h2.y);
+      if constexpr (KEEP) {
+        g2.x = fmaf(a.hw1[k], hk.x, g2.x);
+        g2.y = fmaf(a.hw1[k], hk.y, g2.y);
+      }
     }
     hd[0][c] = h2.x;
     hd[1][c] = h2.y;
+    if constexpr (KEEP) {
+      *reinterpret_cast<float2*>(a.hx0 + c * a.N + idx) = h2;
+      *reinterpret_cast<float2*>(a.hx1 + c * a.N + idx) = g2;
+    }
   }
 }
 
-template <int NH>
+template <int NH, bool KEEP>
 __device__ __forceinline__ void extrap_cell_n(const RowArgs& a, long long idx, float (&hd)[3]) {
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    float h = 0.f;
+    float h = 0.f, g = 0.f;
 #pragma unroll
-    for (int k = 0; k < NH; ++k) h = fmaf(a.hw[k], a.hist[k][c * a.N + idx], h);
+    for (int k = 0; k < NH; ++k) {
+      const float hk = a.hist[k][c * a.N + idx];
+      h = fmaf(a.hw[k], hk, h);
+      if constexpr (KEEP) g = fmaf(a.hw1[k], hk, g);
+    }
     hd[c] = h;
+    if constexpr (KEEP) {
+      a.hx0[c * a.N + idx] = h;
+      a.hx1[c * a.N + idx] = g;
+    }
   }
 }
 
-// nh is 5 (quartic, RK4) or 6 (quintic, RKF5(6)); uniform over the grid.
+// nh is 5 (quartic, RK4), 6 (quintic, RKF5(6)) or 1 (a field kept by an earlier stage); uniform over
+// the grid.
 __device__ __forceinline__ void extrap_pair(const RowArgs& a, long long idx, float (&hd)[2][3]) {
   if (a.nh == 6)
-    extrap_pair_n<6>(a, idx, hd);
+    extrap_pair_n<6, false>(a, idx, hd);
+  else if (a.nh == 1)
+    extrap_pair_n<1, false>(a, idx, hd);
+  else if (a.hx0)
+    extrap_pair_n<5, true>(a, idx, hd);
   else
-    extrap_pair_n<5>(a, idx, hd);
+    extrap_pair_n<5, false>(a, idx, hd);
 }
 
 __device__ __forceinline__ void extrap_cell(const RowArgs& a, long long idx, float (&hd)[3]) {
   if (a.nh == 6)
-    extrap_cell_n<6>(a, idx, hd);
+    extrap_cell_n<6, false>(a, idx, hd);
+  else if (a.nh == 1)
+    extrap_cell_n<1, false>(a, idx, hd);
+  else if (a.hx0)
+    extrap_cell_n<5, true>(a, idx, hd);
   else
-    extrap_cell_n<5>(a, idx, hd);
+    extrap_cell_n<5, false>(a, idx, hd);
 }
 
 // Epilogue of the pair of cells (x0, x0 + 1), x0 even, at linear index idx (row of plane z at
@@ -382,7 +414,7 @@ __host__ __device__ constexpr int io_blocks(int T) { return T >= 768 ? 1 : (T >=
 template <int LX, int RB_, int PREC, int KIND = 0>
 __global__ void __launch_bounds__(3 * RB_ * LX / GBD_E,
                                   KIND == 1 ? io_blocks(3 * RB_ * LX / GBD_E) : min_blocks(3 * RB_ * LX / GBD_E))
-    row_kernel(RowArgs a, const float2* __restrict__ tw) {
+    row_kernel(const __grid_constant__ RowArgs a, const float2* __restrict__ tw) {
   constexpr int RB = RB_;
   constexpr int LINES = 3 * RB;
   constexpr int T = LINES * LX / GBD_E;
