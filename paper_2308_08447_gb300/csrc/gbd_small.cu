@@ -503,8 +503,11 @@ __device__ __forceinline__ void z_in_registers(float2 (&x)[3][PZ / 2], KF kfetch
   }
 }
 
-template <int PZ>
-__global__ void __launch_bounds__(384, PZ >= 16 ? 1 : 2) small_conv_kernel(const __grid_constant__ SmallConvArgs s, const float2* __restrict__ tw) {
+// The z transforms of 16 points take 128 registers or more: TWO runs them at two blocks of 256 threads
+// per SM, otherwise at one of 384.
+__host__ __device__ constexpr int small_conv_threads(int PZ, bool two) { return PZ >= 16 && two ? 256 : 384; }
+template <int PZ, bool TWO = true>
+__global__ void __launch_bounds__(small_conv_threads(PZ, TWO), TWO ? 2 : 1) small_conv_kernel(const __grid_constant__ SmallConvArgs s, const float2* __restrict__ tw) {
   const ColArgs& a = s.a;
   const FftPlan& f = s.f;
   const int T = blockDim.x, tid = threadIdx.x;
@@ -608,9 +611,9 @@ constexpr int kSmallThreads = 384;
 
 // Threads of a block: one per x-row item or y frequency while the blocks leave SMs to spare (96x64x1
 // stage 10.4 -> 9.1 us), else one per eight values (the eight-mesh batch 6620 -> 6370 us).
-static int small_threads(int blocks, int items, int values) {
+static int small_threads(int blocks, int items, int values, int most = kSmallThreads) {
   const int t = blocks <= 2 * kTileBlocks ? items : values / 8;
-  return std::min(kSmallThreads, (t + 31) / 32 * 32);
+  return std::min(most, (t + 31) / 32 * 32);
 }
 
 static size_t small_row_smem(const FftPlan& f, int RB, int nx, int stage_rows) {
@@ -687,13 +690,22 @@ bool launch_small_conv(const ColArgs& a, float2* S, float2* T, int phases, const
   s.phases = phases;
   if (!make_fft_plan(a.Py, s.f)) return false;
   const size_t smem = small_conv_smem(s.f, a.nz);
+  // 5 to 8 layers: two blocks per SM where shared memory and the number of blocks allow (201x117x5 stage
+  // 37.6 -> 33.9 us, 512x128x6 49.8 -> 44.6; 256x256x8, whose lines fill an SM, 49.4 -> 54.1, and
+  // 128x128x8, with fewer blocks than SMs, 24.3 -> 27.2)
+  const bool two = smem <= kSmallSmem / 2 && a.Hx > kTileBlocks;
   const int values = 3 * a.nz * a.Py;
-  const unsigned threads = (unsigned)small_threads(a.Hx, std::max(a.Py, values / 8), values);
+  const unsigned threads = (unsigned)small_threads(a.Hx, std::max(a.Py, values / 8), values, small_conv_threads(a.Pz, two));
   switch (a.Pz) {
     case 1: launch_pdl(small_conv_kernel<1>, a.Hx, threads, smem, st, s, tw); return true;
     case 4: launch_pdl(small_conv_kernel<4>, a.Hx, threads, smem, st, s, tw); return true;
     case 8: launch_pdl(small_conv_kernel<8>, a.Hx, threads, smem, st, s, tw); return true;
-    case 16: launch_pdl(small_conv_kernel<16>, a.Hx, threads, smem, st, s, tw); return true;
+    case 16:
+      if (two)
+        launch_pdl(small_conv_kernel<16, true>, a.Hx, threads, smem, st, s, tw);
+      else
+        launch_pdl(small_conv_kernel<16, false>, a.Hx, threads, smem, st, s, tw);
+      return true;
     default: return false;
   }
 }
@@ -703,7 +715,8 @@ void prepare_small() {
   prep(small_conv_kernel<1>, kSmallSmem);
   prep(small_conv_kernel<4>, kSmallSmem);
   prep(small_conv_kernel<8>, kSmallSmem);
-  prep(small_conv_kernel<16>, kSmallSmem);
+  prep(small_conv_kernel<16, true>, kSmallSmem);
+  prep(small_conv_kernel<16, false>, kSmallSmem);
 }
 
 }  // namespace gbd
