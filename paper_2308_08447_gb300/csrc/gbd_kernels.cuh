@@ -62,11 +62,13 @@ __host__ __device__ constexpr int film_cols(int Py, int v) {
          : v == 0      ? (Py >= 1024 ? 1 : 1024 / Py)
                        : (Py >= 4096 ? 1 : 2 * (Py >= 1024 ? 1 : 1024 / Py));
 }
-// y lines per 3D y-pass block
+// y lines per 3D y-pass block: 128 threads (v = 0; 3 * 2^k and 5 * 2^k: 144 to 192) or 256. The pass
+// runs at 80 % of the L1 data pipe's peak, and smaller blocks keep more of them in different phases
+// (512x512x64 forward 198 -> 175 us, inverse 190 -> 171; 384x384x64 189 -> 141, 141 -> 129).
 __host__ __device__ constexpr int ypass_lines(int Py, int v) {
-  return mixed_len(Py) ? (pow2_floor(Py) >= 4096 ? 1 : 4096 / pow2_floor(Py))
-         : v == 0      ? (Py >= 4096 ? 1 : 4096 / Py)
-                       : (Py >= 2048 ? 1 : 2048 / Py);
+  return mixed_len(Py) ? (pow2_floor(Py) >= 2048 ? 1 : 2048 / pow2_floor(Py))
+         : v == 0      ? (Py >= 2048 ? 1 : 2048 / Py)
+                       : (Py >= 4096 ? 1 : 4096 / Py);
 }
 // (kx, ky) columns per z-convolution block (3 lines each)
 __host__ __device__ constexpr int zconv_cols(int Pz, int v) {
@@ -81,7 +83,7 @@ __host__ __device__ constexpr int film_cols_small(int Py, int prec, int i) {
                        : (Py > 1 && (i == 0 || prec == 0)) ? (1024 / Py) >> (i + 1) : 0;
 }
 __host__ __device__ constexpr int ypass_lines_small(int Py, int i) {
-  return mixed_len(Py) ? (i == 0 ? ypass_lines(Py, 0) / 4 : ypass_lines(Py, 0) / 8) : (2048 / Py) >> (i + 1);
+  return mixed_len(Py) ? (i == 0 ? ypass_lines(Py, 0) / 2 : ypass_lines(Py, 0) / 4) : (2048 / Py) >> (i + 1);
 }
 __host__ __device__ constexpr int zconv_cols_small(int Pz, int prec, int i) {
   return (i == 0 || prec == 0) ? (1024 / Pz) >> (i + 1) : 0;

@@ -72,11 +72,11 @@ template <int L, bool INV, int PREC>
 static void ypass_launch_tile(int var, const ColArgs* a, const float2* tw, cudaStream_t st) {
   constexpr int V0 = ypass_lines(L, 0), V1 = ypass_lines(L, 1);
   constexpr int S0 = ypass_lines_small(L, 0), S1 = ypass_lines_small(L, 1);
-  const int c = a ? pick_tile(a->lines_total, var == 0 ? V0 : V1, V1, S0, S1) : 0;
+  const int c = a ? pick_tile(a->lines_total, var == 0 ? V0 : V1, V0, S0, S1) : 0;
   if (!a || c == V0) ypass_launch_t<L, V0, INV, PREC>(a, tw, st);
   if constexpr (V1 != V0)
     if (!a || c == V1) ypass_launch_t<L, V1, INV, PREC>(a, tw, st);
-  if constexpr (S0 > 0 && S0 != V1)
+  if constexpr (S0 > 0 && S0 != V0)
     if (!a || c == S0) ypass_launch_t<L, S0, INV, PREC>(a, tw, st);
   if constexpr (S1 > 0)
     if (!a || c == S1) ypass_launch_t<L, S1, INV, PREC>(a, tw, st);
