@@ -263,9 +263,13 @@ const char* gbd_last_error(void);
  * row group's inputs into shared memory (cp.async) while it transforms the current group -- in
  * RK stages variant 2 stages the spectrum tile and the field rows (one block per SM), variant 3
  * the spectrum tile only (two blocks per SM; nx a multiple of 64); transform-only launches stage
- * their input (two blocks per SM). They are used where they apply (x transform length Px/2 in
- * [64, 2048], open x axis, nx a multiple of 4, ny a multiple of the group's rows, the staged
- * fields 16-byte aligned; otherwise variant 1 runs). A new mesh starts with variant 1. All variants give identical
+ * their input (two blocks per SM). They are used where they apply (x transform length Px/2 a power
+ * of two in [64, 2048], open x axis, nx a multiple of 4, ny a multiple of the group's rows, the
+ * staged fields 16-byte aligned; otherwise variant 1 runs). A new mesh starts with variant 1. A
+ * variant is the largest tile: a launch that it would spread over fewer blocks than the GPU has
+ * SMs takes a smaller one. Some passes have one kernel whatever the variant: the x rows of small
+ * meshes, of lengths 3 * 2^k and 5 * 2^k and of most 3D meshes, and the convolution along y and z
+ * of small films and of up to 8 layers. All variants give identical
  * results -- each line's FFT and each cell's update do not depend on how lines are grouped --
  * and differ only in speed, which depends on the mesh size. gbd_mesh_autotune times the
  * variants of each pass this mesh uses (on its own buffers, which it zeroes; the stream is
@@ -337,7 +341,8 @@ enum {
  * gbd_mesh_read_timing. GBD_TIMING_NVTX: every launch's enqueue is wrapped in an NVTX range
  * named after its pass class ("row_fwd", "row_inv", "row_rk", "film_conv", "y_fwd", "z_conv",
  * "y_inv", "extrap_stage"), for profilers that filter kernels by NVTX range; the two combine.
- * Batched runs (gbd_batch_run*) are not traced. */
+ * A 3D convolution that runs in one launch (class z_conv) is launched pass by pass, with the same
+ * results, while events are on. Batched runs (gbd_batch_run*) are not traced. */
 #define GBD_TIMING_EVENTS 1
 #define GBD_TIMING_NVTX 2
 gbd_status gbd_mesh_set_timing(gbd_mesh* mesh, int enable);

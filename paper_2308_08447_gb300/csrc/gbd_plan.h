@@ -10,7 +10,7 @@ namespace gbd {
 constexpr int kMaxPad = 4096;
 constexpr int kMaxPadX = 8192;
 // Transform lengths 3 * 2^k and 5 * 2^k with kernels (FP32): the half length Lx = Px / 2 of
-// the x transform and the y length Py may take these values (gbd_mixed_row.cu,
+// the x transform and the y length Py may take these values (gbd_rowpair_mixed.cu,
 // gbd_mixed_conv.cu); every other length is a power of two.
 constexpr int kMixedLens[] = {96, 160, 192, 320, 384, 640, 768, 1280, 1536, 2560, 3072};
 

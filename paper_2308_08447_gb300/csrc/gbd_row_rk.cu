@@ -1,6 +1,7 @@
 // Staged RK-stage x-row kernels (Sec. II, Eq. 1 and Sec. III: the inverse x transform, the
 // exchange + LLG + RK4 stage epilogue and the next stage's forward x transform): the FP32 row
-// kernel's KIND 2 instances for the power-of-two lengths whose tile takes the staged epilogue,
+// kernel's KIND 2 instances for the power-of-two lengths from 1024 (below, the launches that fill their
+// tile take the paired kernel) whose tile takes the staged epilogue,
 // compiled without the branches those launches never take. Their own translation unit, built in
 // parallel with the others.
 #include "gbd_row.cuh"
@@ -20,14 +21,14 @@ bool row_rk_dispatch(int Lx, int RB, const RowArgs* a, const float2* tw, cudaStr
   row_switch(Lx, [&](auto lx) {
     constexpr int LX = decltype(lx)::value;
     constexpr int R0 = row_rb(LX, 0), R1 = row_rb(LX, 1);
-    if constexpr (row_stage_ok<LX, R0, 0>()) {
+    if constexpr (LX >= 1024 && row_stage_ok<LX, R0, 0>()) {
       if (RB == R0) {
         row_rk_launch_t<LX, R0>(a, tw, st);
         done = true;
         return;
       }
     }
-    if constexpr (R1 != R0 && row_stage_ok<LX, R1, 0>()) {
+    if constexpr (LX >= 1024 && R1 != R0 && row_stage_ok<LX, R1, 0>()) {
       if (RB == R1) {
         row_rk_launch_t<LX, R1>(a, tw, st);
         done = true;

@@ -28,11 +28,8 @@ namespace gbd {
 // leaves room for two blocks per SM.
 enum PipeKind : int { PIPE_FWD = 0, PIPE_INV = 1, PIPE_RK = 2, PIPE_RKS = 3 };
 
-// rows per group: 2048 complex values per component (LX in [64, 2048]); for LX = 3 * 2^k or
-// 5 * 2^k, 2048 over the next power of two above LX
-__host__ __device__ constexpr int pipe_rb(int LX) {
-  return mixed_len(LX) ? (2048 / (2 * pow2_floor(LX)) > 0 ? 2048 / (2 * pow2_floor(LX)) : 1) : (LX >= 2048 ? 1 : 2048 / LX);
-}
+// rows per group: 2048 complex values per component (LX in [64, 2048])
+__host__ __device__ constexpr int pipe_rb(int LX) { return LX >= 2048 ? 1 : 2048 / LX; }
 
 // Shared-memory layout of the pipelined kernel, in float2 slots, each part starting on a
 // 16-byte boundary: the lines, the staged spectrum tile [3][LX + 1][RB] (not for forward-only
@@ -414,12 +411,11 @@ static int pipe_kind(int Lx, const RowArgs& a, int var) {
   return -1;
 }
 
-// Launches (a == nullptr: prepares every kind) the pipelined kernel for length Lx through the
-// length switch SW (row_switch, or the mixed-length one); false when there is no
-// instantiation for Lx.
-template <class SW>
-static bool pipe_dispatch_with(SW sw, int Lx, int kind, const RowArgs* a, const float2* tw, cudaStream_t st) {
-  auto go = [&](auto lx) {
+// Launches (a == nullptr: prepares every kind) the pipelined kernel for length Lx; false when there is
+// no instantiation for Lx.
+static bool pipe_dispatch(int Lx, int kind, const RowArgs* a, const float2* tw, cudaStream_t st) {
+  if (Lx < 64 || Lx > 2048) return false;
+  return row_switch(Lx, [&](auto lx) {
     constexpr int LX = decltype(lx)::value;
     if constexpr (LX >= 64 && LX <= 2048) {
       if (kind < 0 || kind == PIPE_FWD) pipe_launch_t<LX, PIPE_FWD>(a, tw, st);
@@ -427,12 +423,7 @@ static bool pipe_dispatch_with(SW sw, int Lx, int kind, const RowArgs* a, const 
       if (kind < 0 || kind == PIPE_RK) pipe_launch_t<LX, PIPE_RK>(a, tw, st);
       if (kind < 0 || kind == PIPE_RKS) pipe_launch_t<LX, PIPE_RKS>(a, tw, st);
     }
-  };
-  if (Lx < 64 || Lx > 2048) return false;
-  return sw(Lx, go);
-}
-static bool pipe_dispatch(int Lx, int kind, const RowArgs* a, const float2* tw, cudaStream_t st) {
-  return pipe_dispatch_with([](int L, auto f) { return row_switch(L, f); }, Lx, kind, a, tw, st);
+  });
 }
 
 }  // namespace gbd

@@ -659,7 +659,9 @@ bool launch_small_row(int Lx, const RowArgs& a, const float2* tw, cudaStream_t s
   s.staged = 0;
   if (small_stage_applies(a, RB) && smem_of(1) <= kSmallSmem) {
     s.staged = 1;
-    if (a.mode != ROW_RK1 && smem_of(s.staged | 4) <= kSmallSmem / 2) s.staged |= 4;
+    // (not where the next stage's input replaces m0: the autotuner's repeated launch, without a
+    // convolution in between, would read what the launch before writes)
+    if (a.mode != ROW_RK1 && a.m0 != a.mnext && smem_of(s.staged | 4) <= kSmallSmem / 2) s.staged |= 4;
     if (a.nz > 1 && smem_of(s.staged | 2) <= kSmallSmem / 2) s.staged |= 2;
   }
   const size_t smem = smem_of(s.staged);
