@@ -117,6 +117,10 @@ __device__ __forceinline__ cpair cmul(cpair a, float2 w) {
   const float2 wx = pdup(w.x), wy = pdup(w.y);
   return {pfma(a.x, wx, pneg(pmul(a.y, wy))), pfma(a.x, wy, pmul(a.y, wx))};
 }
+__device__ __forceinline__ cpair cmul(float2 w, cpair a) {   // rounds as cmul(float2 w, float2 a)
+  const float2 wx = pdup(w.x), wy = pdup(w.y);
+  return {pfma(wx, a.x, pneg(pmul(wy, a.y))), pfma(wx, a.y, pmul(wy, a.x))};
+}
 __device__ __forceinline__ cpair cscale(cpair a, float s) { return {pmul(a.x, pdup(s)), pmul(a.y, pdup(s))}; }
 __device__ __forceinline__ cpair cfma(float s, cpair a, cpair b) { return {pfma(pdup(s), a.x, b.x), pfma(pdup(s), a.y, b.y)}; }
 template <int S>

@@ -134,6 +134,8 @@ static bool transform_only(const RowArgs& a) { return a.mode == ROW_FWD || (a.mo
 //     / 193, 512x1024x1 43 / 39; shorter films 512x512x1 21 / 23);
 //   - below, epilogues: 3D meshes and films that give 90 blocks (480x240x2 39 / 34, 512x512x1 30 / 27,
 //     400x400x1 30 / 26; 256x512x1 15 / 17).
+// The rule may differ by mode where L is a power of two only: there both kernels round alike, so that a
+// run split over calls, whose first forward rows are a launch of their own, equals the unsplit run.
 static bool take_pair(int Lx, const RowArgs& a) {
   if (mixed_len(Lx)) return true;
   if ((a.per & 1) || Lx < 32) return false;

@@ -7,6 +7,8 @@
 // value, at the same FMA-pipe time. A block takes NPR row pairs (three pair lines each) and
 // 3 NPR L / 16 threads of 16 pair values. Rows are paired along the flattened (z, y) index; a pair's
 // spectrum is one 16-byte vector of the [kx][y] spectrum where the two rows are adjacent there.
+// For powers of two every operation rounds as row_kernel's, so that a mesh may run its transforms
+// in one kernel and its stages in the other: a run split over calls equals the unsplit run.
 #pragma once
 #include "gbd_row.cuh"
 
@@ -234,11 +236,10 @@ __global__ void __launch_bounds__(pair_threads(L, NPR), pair_blocks(pair_threads
         const cpair s1 = cadd(A[i], conj(B[i])), d1 = csub(A[i], conj(B[i]));
         if (i == 0 && jj == 0) {
           tl[pad(0)] = cadd_i<1>(s1, d1);
-          // k = L/2: W^(L/2) = -i, so Z = 2 conj(X)
-          tl[pad(HALF)] = conj(cadd(M, M));
+          tl[pad(HALF)] = cadd_i<1>(cadd(M, conj(M)), cmul(cconj(twiddle_at<-1>(tw, 2 * L, HALF)), csub(M, conj(M))));
         } else {
           // with t = W^-k (A - B*): Z[k] = s1 + i t, Z[L - k] = (s1 - i t)*
-          const cpair t = cmul(d1, cconj(wp));
+          const cpair t = cmul(cconj(wp), d1);
           tl[pad(k)] = cadd_i<1>(s1, t);
           tl[pad(L - k)] = conj(cadd_i<-1>(s1, t));
         }
@@ -451,14 +452,16 @@ __global__ void __launch_bounds__(pair_threads(L, NPR), pair_blocks(pair_threads
       const float2 zero = make_float2(0.f, 0.f);
       sstore(oa, {padd(A.x, A.y), zero});   // X[0]
       sstore(ob, {psub(A.x, A.y), zero});   // X[L]
-      sstore((long long)HALF * ny, conj(tl[pad(HALF)]));
+      const cpair Mz = tl[pad(HALF)];       // X[L/2], of one Z
+      sstore((long long)HALF * ny,
+             cscale(cadd_i<-1>(cadd(Mz, conj(Mz)), cmul(twiddle_at<-1>(tw, 2 * L, HALF), csub(Mz, conj(Mz)))), 0.5f));
     } else {
       const cpair B = tl[pad(L - k)];
       const float2 wp = twiddle_at<-1>(tw, 2 * L, k);
-      // with s = (A + B*)/2, t = W^k (A - B*)/2: X[k] = s - i t, X[L - k] = (s + i t)*
-      const cpair s1 = cscale(cadd(A, conj(B)), 0.5f), t = cscale(cmul(csub(A, conj(B)), wp), 0.5f);
-      sstore(oa, cadd_i<-1>(s1, t));
-      sstore(ob, conj(cadd_i<1>(s1, t)));
+      // with s = A + B*, t = W^k (A - B*): X[k] = (s - i t)/2, X[L - k] = ((s + i t)/2)*
+      const cpair s1 = cadd(A, conj(B)), t = cmul(wp, csub(A, conj(B)));
+      sstore(oa, cscale(cadd_i<-1>(s1, t), 0.5f));
+      sstore(ob, conj(cscale(cadd_i<1>(s1, t), 0.5f)));
     }
   }
 }

@@ -62,3 +62,20 @@ def test_z_lengths(g, n):
     mesh.demag(to_dev(M), H)
     assert e_inf(to_host(H), C.fft_conv(M.astype(np.float64), T.tensor_all_offsets(n, CELL))) <= TOL_FP32
     mesh.close()
+
+
+@pytest.mark.parametrize("n", [(512, 400, 1), (400, 400, 1), (256, 800, 1), (800, 300, 1), (1024, 96, 1), (512, 1030, 1),
+                               (300, 420, 1), (128, 64, 8), (250, 61, 3)])
+def test_split_calls_equal_one_call(g, n):
+    # a call's first forward transform, its stages and its last stage may run in different kernels:
+    # their results are bit-identical
+    import torch
+    m = to_dev(W.vortex_noise(n, CELL, 11))
+    mesh = g.Mesh(n, CELL, MS, A_ex=A, alpha=ALPHA)
+    one, split = m.clone(), m.clone()
+    mesh.llg_step(one, 6, DT)
+    for k in (1, 2, 3):
+        mesh.llg_step(split, k, DT)
+    torch.cuda.synchronize()
+    assert torch.equal(one, split)
+    mesh.close()
