@@ -275,7 +275,7 @@ const char* gbd_last_error(void);
  * variants of each pass this mesh uses (on its own buffers, which it zeroes; the stream is
  * synchronized) and keeps the fastest; results are cached per (nx, ny, nz, device) in the
  * process and, when the environment variable GBD_AUTOTUNE_CACHE names a file, in that text
- * file. Requires gbd_set_kernel. Variants (row, film, y, z): row 0 to 3, the others 0 or 1.
+ * file (choices that a version with other kernels wrote there are passed over). Requires gbd_set_kernel. Variants (row, film, y, z): row 0 to 3, the others 0 or 1.
  * The autotuner also chooses the padded lengths: a mesh planned with a 3 * 2^k or 5 * 2^k
  * length (see GBD_FLAG_POW2_PAD) is timed against the same mesh on power-of-two lengths (a
  * scratch twin with its own tuned tiles), and moves onto the power-of-two plan when that is

@@ -1479,8 +1479,9 @@ extern "C" gbd_status gbd_demag_noalloc(gbd_mesh* m, const float* M, float* H, v
 // are grouped into blocks -- so the choice only changes speed. gbd_mesh_autotune times both
 // shapes of each pass the mesh uses, on the mesh's own (zeroed) buffers, keeps the faster one,
 // and caches the choice by mesh size and device: in the process, and in the text file named
-// by GBD_AUTOTUNE_CACHE when that is set (lines "nx ny nz device Px Py precision var_row var_film
-// var_y var_z pow2 var_row_io"). For a mesh planned with 3 * 2^k / 5 * 2^k lengths it also times the
+// by GBD_AUTOTUNE_CACHE when that is set (lines "gbd<generation> nx ny nz device Px Py precision var_row
+// var_film var_y var_z pow2 var_row_io"). A choice holds for the kernels it was timed on: lines of
+// another generation, and the lines without one that older versions wrote, are passed over. For a mesh planned with 3 * 2^k / 5 * 2^k lengths it also times the
 // power-of-two plan of the same mesh and moves the mesh onto it when that is faster (pow2 = 1).
 
 namespace {
@@ -1499,6 +1500,9 @@ struct TuneKey {
 std::mutex g_tune_mu;
 std::map<TuneKey, std::array<int, 6>> g_tune;   // variants (row, film, y, z), power-of-two padding, row (transforms only)
 bool g_tune_file_read = false;
+// Raised whenever a variant number comes to mean another tile or kernel, or the kernels that a mesh
+// runs change (without it: y variants 0 and 1 the other way round).
+constexpr int kTuneGeneration = 2;
 
 const char* tune_file() {
   const char* p = std::getenv("GBD_AUTOTUNE_CACHE");
@@ -1512,10 +1516,14 @@ void read_tune_file_locked() {
   if (!path) return;
   FILE* f = std::fopen(path, "r");
   if (!f) return;
-  TuneKey k;
-  std::array<int, 6> v;
-  while (std::fscanf(f, "%d %d %d %d %d %d %d %d %d %d %d %d %d", &k.nx, &k.ny, &k.nz, &k.dev, &k.Px, &k.Py, &k.prec,
-                     &v[0], &v[1], &v[2], &v[3], &v[4], &v[5]) == 13) {
+  char line[256];
+  while (std::fgets(line, sizeof line, f)) {
+    int gen = 0;
+    TuneKey k;
+    std::array<int, 6> v;
+    if (std::sscanf(line, "gbd%d %d %d %d %d %d %d %d %d %d %d %d %d %d", &gen, &k.nx, &k.ny, &k.nz, &k.dev, &k.Px, &k.Py,
+                    &k.prec, &v[0], &v[1], &v[2], &v[3], &v[4], &v[5]) != 14 || gen != kTuneGeneration)
+      continue;
     bool ok = (v[4] == 0 || v[4] == 1) && v[5] >= 0 && v[5] <= 3;
     for (int i = 0; i < 4; ++i) ok = ok && (v[i] == 0 || v[i] == 1 || (i == 0 && (v[i] == 2 || v[i] == 3)));
     if (ok) g_tune[k] = v;
@@ -1528,8 +1536,8 @@ void append_tune_file_locked(const TuneKey& k, const std::array<int, 6>& v) {
   if (!path) return;
   FILE* f = std::fopen(path, "a");
   if (!f) return;
-  std::fprintf(f, "%d %d %d %d %d %d %d %d %d %d %d %d %d\n", k.nx, k.ny, k.nz, k.dev, k.Px, k.Py, k.prec, v[0], v[1],
-               v[2], v[3], v[4], v[5]);
+  std::fprintf(f, "gbd%d %d %d %d %d %d %d %d %d %d %d %d %d %d\n", kTuneGeneration, k.nx, k.ny, k.nz, k.dev, k.Px, k.Py,
+               k.prec, v[0], v[1], v[2], v[3], v[4], v[5]);
   std::fclose(f);
 }
 
