@@ -1650,6 +1650,7 @@ gbd_status move_to_pow2(gbd_mesh* m, void* stream) {
   std::swap(m->T, twin->T);
   std::swap(m->K, twin->K);
   std::swap(m->tw, twin->tw);
+  std::swap(m->status, twin->status);   // the status word lies behind the twiddles
   m->d.flags |= GBD_FLAG_POW2_PAD;
   ++m->version;
   gbd_mesh_destroy(twin);
