@@ -108,6 +108,10 @@ __device__ __forceinline__ float2 cmul_i(float2 a) {  // a * (S i)
   return S > 0 ? make_float2(-a.y, a.x) : make_float2(a.y, -a.x);
 }
 template <int S>
+__device__ __forceinline__ float2 cfma_i(float s, float2 a, float2 b) {  // S i s a + b
+  return make_float2(fmaf(-S * s, a.y, b.x), fmaf(S * s, a.x, b.y));
+}
+template <int S>
 __device__ __forceinline__ float2 cadd_i(float2 a, float2 b) {  // a + S i b
   return S > 0 ? make_float2(a.x - b.y, a.y + b.x) : make_float2(a.x + b.y, a.y - b.x);
 }
@@ -126,6 +130,10 @@ __device__ __forceinline__ cpair cfma(float s, cpair a, cpair b) { return {pfma(
 template <int S>
 __device__ __forceinline__ cpair cmul_i(cpair a) {
   return S > 0 ? cpair{pneg(a.y), a.x} : cpair{a.y, pneg(a.x)};
+}
+template <int S>
+__device__ __forceinline__ cpair cfma_i(float s, cpair a, cpair b) {
+  return {pfma(pdup(-S * s), a.y, b.x), pfma(pdup(S * s), a.x, b.y)};
 }
 template <int S>
 __device__ __forceinline__ cpair cadd_i(cpair a, cpair b) {
@@ -260,11 +268,11 @@ __device__ __forceinline__ void dft16(V* x) {
 template <int S, class V>
 __device__ __forceinline__ void dft3(V* x) {
   const float h = 0.86602540378443864676f;   // sin(2 pi / 3)
-  const V t1 = cadd(x[1], x[2]), u = cscale(csub(x[1], x[2]), h);
+  const V t1 = cadd(x[1], x[2]), t2 = csub(x[1], x[2]);
   const V m = cfma(-0.5f, t1, x[0]);
   x[0] = cadd(x[0], t1);
-  x[1] = cadd_i<S>(m, u);
-  x[2] = cadd_i<-S>(m, u);
+  x[1] = cfma_i<S>(h, t2, m);
+  x[2] = cfma_i<-S>(h, t2, m);
 }
 
 // DFT_5 by the symmetric pairs a_n = x_n + x_(5-n), b_n = x_n - x_(5-n) (n = 1, 2), with

@@ -17,58 +17,72 @@
 // The arithmetic does not depend on the tile variant or on how the rows are grouped.
 #include <algorithm>
 #include <cstdint>
+#include <type_traits>
 
 #include "gbd_row.cuh"
 
 namespace gbd {
 
-// Radix passes of length L = r 2^k (r in {1, 3, 5}, 2^k >= 16): radix 8 (4, 2) passes and the
-// odd radix last, so that Ns is a power of two in every pass.
+// Radix passes of length L = r 2^k (r in {1, 3, 5}, 2^k >= 16): the odd radix, as in the other kernels,
+// then radix 8 and 4. (The odd radix last keeps Ns a power of two, but costs accuracy: 150x150x6 field,
+// rms error 1.57e-7 against 1.30e-7.)
 struct FftPlan {
   int L, np;
   int ls;                    // float2 slots per line
   int radix[6], ns[6];
   int twoff[6];              // first of the pass's twiddles in the shared table
+  unsigned kdiv[6];          // floor(j / Ns) = umulhi(j, kdiv) for j < 2^16 (0: Ns = 1)
   unsigned mdiv[6];          // floor(b / (L / R)) = umulhi(b, mdiv) for b < 2^16
   int ntw;                   // shared twiddles of all passes
 };
+// Element i of a line sits at i + i / 16, or, where the first radix is odd (ODD), at i: the writes of a
+// first pass of radix 8 or 4 then miss each other's banks, and so do those of radix 3 or 5, of which the
+// pad would put five into one bank (320x320x4 field 64.9 -> 62.9 us).
+template <bool ODD>
+__host__ __device__ __forceinline__ constexpr int at(int i) {
+  return ODD ? i : i + (i >> 4);
+}
 static unsigned magic_div(unsigned d) { return d <= 1 ? 0u : (unsigned)((0x100000000ull + d - 1) / d); }
 __device__ __forceinline__ int fast_div(int b, unsigned m) { return m ? (int)__umulhi((unsigned)b, m) : b; }
-
-__host__ __device__ constexpr int tw_powers(int R) { return R == 8 || R == 5 ? 3 : 2; }
 
 static bool make_fft_plan(int L, FftPlan& f) {
   const int r = odd_part(L);
   if (L < 16 || r > 5 || (r > 1 && L / r < 16)) return false;
   f.L = L;
   f.np = 0;
+  if (r > 1) f.radix[f.np++] = r;
   int k = ilog2(L / r);
   while (k > 0) {
     const int b = (k == 4 || k == 2) ? 2 : 3;   // k >= 4: ends 8, 8 4 or 4 4, never with a radix 2
     f.radix[f.np++] = 1 << b;
     k -= b;
   }
-  if (r > 1) f.radix[f.np++] = r;
   int ns = 1, off = 0;
   for (int p = 0; p < f.np; ++p) {
     f.ns[p] = ns;
     f.twoff[p] = off;
-    if (p > 0) off += tw_powers(f.radix[p]) * ns;
+    if (p > 0) off += (f.radix[p] - 1) * ns;
     f.mdiv[p] = magic_div(L / f.radix[p]);
+    f.kdiv[p] = magic_div(ns);
     ns *= f.radix[p];
   }
   f.ntw = off;
-  f.ls = (L + L / 16) | 1;
+  f.ls = (r > 1 ? at<true>(L) : at<false>(L)) | 1;
   return true;
 }
 
-// Copies the passes' twiddles into shared memory: pass p holds w^e, e = 1, 2 (, 4), at
-// [e][k], w = exp(-2 pi i / (Ns R)).
+// Copies the passes' twiddles into shared memory: pass p holds w^e, 0 < e < R, at [e - 1][k], w =
+// exp(-2 pi i / (Ns R)). Every power comes from the table: products of powers (three loads instead of
+// seven for R = 8) add their own roundings (32x32x8 field, rms error 1.89e-7 against 1.55e-7) at the same
+// time.
 __device__ __forceinline__ void load_twiddles(const FftPlan& f, float2* stw, const float2* __restrict__ tw) {
   for (int p = 1; p < f.np; ++p) {
-    const int R = f.radix[p], ns = f.ns[p], n = tw_powers(R) * ns, sh = 31 - __clz(ns);
+    const int R = f.radix[p], ns = f.ns[p], n = (R - 1) * ns;
     const float2* lev = tw + tw_base(ns * R);
-    for (int i = threadIdx.x; i < n; i += blockDim.x) stw[f.twoff[p] + i] = __ldg(lev + ((i & (ns - 1)) << (i >> sh)));
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+      const int e = fast_div(i, f.kdiv[p]);
+      stw[f.twoff[p] + i] = __ldg(lev + (i - e * ns) * (e + 1));
+    }
   }
 }
 
@@ -77,26 +91,11 @@ __device__ __forceinline__ void prefetch_l1(const void* p) { asm volatile("prefe
 // One radix-R butterfly: twiddles from the shared table (sign S), DFT.
 template <int S, int R>
 __device__ __forceinline__ void small_butterfly(float2* v, const float2* __restrict__ t, int k, int ns) {
-  auto w = [&](int e) {
-    const float2 x = t[e * ns + k];
-    return S < 0 ? x : cconj(x);
-  };
   if (ns > 1) {
-    const float2 w1 = w(0), w2 = w(1);
-    v[1] = cmul(v[1], w1);
-    v[2] = cmul(v[2], w2);
-    if constexpr (R > 3) {
-      const float2 w3 = cmul(w1, w2);
-      v[3] = cmul(v[3], w3);
-      if constexpr (R > 4) {
-        const float2 w4 = w(2);
-        v[4] = cmul(v[4], w4);
-        if constexpr (R > 5) {
-          v[5] = cmul(v[5], cmul(w1, w4));
-          v[6] = cmul(v[6], cmul(w2, w4));
-          v[7] = cmul(v[7], cmul(w3, w4));
-        }
-      }
+#pragma unroll
+    for (int e = 1; e < R; ++e) {
+      const float2 w = t[(e - 1) * ns + k];
+      v[e] = cmul(v[e], S < 0 ? w : cconj(w));
     }
   }
   dft<R, S>(v);
@@ -104,13 +103,13 @@ __device__ __forceinline__ void small_butterfly(float2* v, const float2* __restr
 
 // Pass p over `lines` lines: LD(line, i) -> element i, ST(line, i, v). Stockham: reads j + r L/R,
 // writes (j - k) R + k + q Ns.
-template <int S, int R, class LD, class ST>
+template <int S, int R, bool ODD, class LD, class ST>
 __device__ __forceinline__ void small_pass_r(const FftPlan& f, int p, int lines, const float2* __restrict__ stw, LD ld, ST st) {
   const int LR = f.L / R, ns = f.ns[p];
   for (int b = threadIdx.x; b < lines * LR; b += blockDim.x) {
     const int line = fast_div(b, f.mdiv[p]);
     const int j = b - line * LR;
-    const int k = j & (ns - 1);
+    const int k = ODD ? j - fast_div(j, f.kdiv[p]) * ns : j & (ns - 1);
     float2 v[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) v[r] = ld(line, j + r * LR);
@@ -120,26 +119,29 @@ __device__ __forceinline__ void small_pass_r(const FftPlan& f, int p, int lines,
     for (int q = 0; q < R; ++q) st(line, base + q * ns, v[q]);
   }
 }
-template <int S, class LD, class ST>
+template <int S, bool ODD, class LD, class ST>
 __device__ __forceinline__ void small_pass(const FftPlan& f, int p, int lines, const float2* __restrict__ stw, LD ld, ST st) {
-  switch (f.radix[p]) {
-    case 8: small_pass_r<S, 8>(f, p, lines, stw, ld, st); break;
-    case 3: small_pass_r<S, 3>(f, p, lines, stw, ld, st); break;
-    case 5: small_pass_r<S, 5>(f, p, lines, stw, ld, st); break;
-    default: small_pass_r<S, 4>(f, p, lines, stw, ld, st); break;
-  }
+  const int R = f.radix[p];
+  if (R == 8)
+    small_pass_r<S, 8, ODD>(f, p, lines, stw, ld, st);
+  else if (!ODD || R == 4)
+    small_pass_r<S, 4, ODD>(f, p, lines, stw, ld, st);
+  else if (R == 3)
+    small_pass_r<S, 3, ODD>(f, p, lines, stw, ld, st);
+  else
+    small_pass_r<S, 5, ODD>(f, p, lines, stw, ld, st);
 }
 // Passes [p0, p1) between the buffers, starting from x; returns the buffer that holds the result.
 // A barrier precedes each pass.
-template <int S>
+template <int S, bool ODD>
 __device__ __forceinline__ float2* small_passes(const FftPlan& f, int p0, int p1, int lines, const float2* __restrict__ stw,
                                                 float2* x, float2* y) {
   for (int p = p0; p < p1; ++p) {
     __syncthreads();
     const float2* src = x;
     float2* dst = y;
-    small_pass<S>(f, p, lines, stw, [&](int l, int i) { return src[l * f.ls + pad(i)]; },
-                  [&](int l, int i, float2 v) { dst[l * f.ls + pad(i)] = v; });
+    small_pass<S, ODD>(f, p, lines, stw, [&](int l, int i) { return src[l * f.ls + at<ODD>(i)]; },
+                  [&](int l, int i, float2 v) { dst[l * f.ls + at<ODD>(i)] = v; });
     y = x;
     x = dst;
   }
@@ -166,6 +168,8 @@ __host__ __device__ __forceinline__ int small_stage_rows(int RB, int staged) {
   return (staged & 1) ? RB + 2 + ((staged & 2) ? 2 * RB : 0) + ((staged & 4) ? 2 * RB : 0) : 0;
 }
 
+// ODD: Lx is 3 * 2^k or 5 * 2^k.
+template <bool ODD>
 __global__ void __launch_bounds__(384, 2) small_row_kernel(const __grid_constant__ SmallRowArgs s, const float2* __restrict__ tw) {
   const RowArgs& a = s.a;
   const FftPlan& f = s.f;
@@ -264,16 +268,16 @@ __global__ void __launch_bounds__(384, 2) small_row_kernel(const __grid_constant
           const float2 Au = A[i], Bu = B[i];
           float2* D = X + (c * RB + rr) * f.ls;
           if (k == 0) {
-            D[pad(0)] = cadd(cadd(Au, cconj(Bu)), cmul_i<1>(csub(Au, cconj(Bu))));
+            D[at<ODD>(0)] = cadd(cadd(Au, cconj(Bu)), cmul_i<1>(csub(Au, cconj(Bu))));
           } else {
-            D[pad(k)] = cadd(cadd(Au, cconj(Bu)), cmul_i<1>(cmul(wm, csub(Au, cconj(Bu)))));
-            if (k != L - k) D[pad(L - k)] = csub(cadd(Bu, cconj(Au)), cmul_i<1>(cmul(wp, csub(Bu, cconj(Au)))));
+            D[at<ODD>(k)] = cadd(cadd(Au, cconj(Bu)), cmul_i<1>(cmul(wm, csub(Au, cconj(Bu)))));
+            if (k != L - k) D[at<ODD>(L - k)] = csub(cadd(Bu, cconj(Au)), cmul_i<1>(cmul(wp, csub(Bu, cconj(Au)))));
           }
         }
       }
     }
     // 2. unnormalised inverse FFT
-    float2* R = small_passes<1>(f, 0, f.np, lines, stw, X, Y);
+    float2* R = small_passes<1, ODD>(f, 0, f.np, lines, stw, X, Y);
     if (R != X) {
       Y = X;
       X = R;
@@ -282,7 +286,7 @@ __global__ void __launch_bounds__(384, 2) small_row_kernel(const __grid_constant
   }
   if (mode != ROW_FWD) {
     if (s.staged && !mbar_wait(sbar, 0, GBD_WAIT_LIMIT_NS) && a.status) atomicOr(a.status, GBD_DEV_WAIT_TIMEOUT);
-    // 3. epilogue; element x of a row is float 2 pad(x / 2) + (x & 1) of its line
+    // 3. epilogue; element x of a row is float 2 at<ODD>(x / 2) + (x & 1) of its line
     if (s.staged) {
       const int NP2 = nx / 2;
       const long long sz = (long long)nx * ny;
@@ -294,7 +298,7 @@ __global__ void __launch_bounds__(384, 2) small_row_kernel(const __grid_constant
         float hd[2][3], mv[2][3], lap[2][3], m0v[2][3] = {}, accv[2][3] = {}, mn[2][3], ao[2][3], res[2][3];
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-          const float2 h2 = X[(c * RB + rr) * f.ls + pad(xp)];
+          const float2 h2 = X[(c * RB + rr) * f.ls + at<ODD>(xp)];
           hd[0][c] = h2.x * a.hscale;
           hd[1][c] = h2.y * a.hscale;
           if (a.hrec) *reinterpret_cast<float2*>(a.hrec + c * N + idx) = make_float2(hd[0][c], hd[1][c]);
@@ -335,7 +339,7 @@ __global__ void __launch_bounds__(384, 2) small_row_kernel(const __grid_constant
             *reinterpret_cast<float2*>(a.acc + c * N + idx) = make_float2(ao[0][c], ao[1][c]);
             *reinterpret_cast<float2*>(a.mnext + c * N + idx) = v;
           }
-          X[(c * RB + rr) * f.ls + pad(xp)] = v;
+          X[(c * RB + rr) * f.ls + at<ODD>(xp)] = v;
         }
       }
     } else if (mode == ROW_H) {
@@ -343,7 +347,7 @@ __global__ void __launch_bounds__(384, 2) small_row_kernel(const __grid_constant
         const int line = fast_div(e, s.mnx), x = e - line * nx;
         const int rr = line & (RB - 1), c = line >> s.rb_log;
         if (r0 + rr >= a.rows) continue;
-        const float v = reinterpret_cast<const float*>(X + line * f.ls)[2 * pad(x >> 1) + (x & 1)] * a.hscale;
+        const float v = reinterpret_cast<const float*>(X + line * f.ls)[2 * at<ODD>(x >> 1) + (x & 1)] * a.hscale;
         const long long idx = c * N + (long long)(r0 + rr) * nx + x;
         if (a.hrec) a.hrec[idx] = v;
         a.out[idx] = v;
@@ -362,14 +366,14 @@ __global__ void __launch_bounds__(384, 2) small_row_kernel(const __grid_constant
         } else {
 #pragma unroll
           for (int c = 0; c < 3; ++c) {
-            const float2 h2 = X[(c * RB + rr) * f.ls + pad(xp)];
+            const float2 h2 = X[(c * RB + rr) * f.ls + at<ODD>(xp)];
             hd[0][c] = h2.x * a.hscale;
             hd[1][c] = h2.y * a.hscale;
           }
         }
         if (epilogue_pair<false>(a, mode, z, y, idx, 2 * xp, 0, hd, mn) && a.fwd_after) {
 #pragma unroll
-          for (int c = 0; c < 3; ++c) X[(c * RB + rr) * f.ls + pad(xp)] = make_float2(mn[0][c], mn[1][c]);
+          for (int c = 0; c < 3; ++c) X[(c * RB + rr) * f.ls + at<ODD>(xp)] = make_float2(mn[0][c], mn[1][c]);
         }
       }
     } else {
@@ -379,7 +383,7 @@ __global__ void __launch_bounds__(384, 2) small_row_kernel(const __grid_constant
         int z, y;
         row_zy(rr, z, y);
         const long long idx = (long long)(r0 + rr) * nx + x;
-        const int fpos = 2 * pad(x >> 1) + (x & 1);
+        const int fpos = 2 * at<ODD>(x >> 1) + (x & 1);
         float hd[3], mn[3];
         if (a.extrap) {
           extrap_cell(a, idx, hd);
@@ -400,7 +404,7 @@ __global__ void __launch_bounds__(384, 2) small_row_kernel(const __grid_constant
       const int rr = line & (RB - 1), c = line >> s.rb_log;
       float v = 0.f;
       if (r0 + rr < a.rows) v = a.in[c * N + (long long)(r0 + rr) * nx + x];
-      reinterpret_cast<float*>(X + line * f.ls)[2 * pad(x >> 1) + (x & 1)] = v;
+      reinterpret_cast<float*>(X + line * f.ls)[2 * at<ODD>(x >> 1) + (x & 1)] = v;
     }
   }
   // 4. zeros beyond the data: up to the middle of the line (open x; the first pass takes the upper
@@ -408,22 +412,22 @@ __global__ void __launch_bounds__(384, 2) small_row_kernel(const __grid_constant
   if (const int pad_x = (xper ? 2 * L : L) - nx; pad_x > 0)
     for (int e = tid; e < lines * pad_x; e += T) {
       const int line = fast_div(e, s.mpad), x = nx + e - line * pad_x;
-      reinterpret_cast<float*>(X + line * f.ls)[2 * pad(x >> 1) + (x & 1)] = 0.f;
+      reinterpret_cast<float*>(X + line * f.ls)[2 * at<ODD>(x >> 1) + (x & 1)] = 0.f;
     }
   if (r0 + RB > a.rows)
     for (int line = 0; line < lines; ++line)
       if (r0 + (line & (RB - 1)) >= a.rows)
-        for (int x = tid; x < nx; x += T) reinterpret_cast<float*>(X + line * f.ls)[2 * pad(x >> 1) + (x & 1)] = 0.f;
+        for (int x = tid; x < nx; x += T) reinterpret_cast<float*>(X + line * f.ls)[2 * at<ODD>(x >> 1) + (x & 1)] = 0.f;
   __syncthreads();
   // 5. forward FFT
   {
     const float2* src = X;
     float2* dst = Y;
-    small_pass<-1>(f, 0, lines, stw,
-                   [&](int l, int i) { return (xper || i < HALF) ? src[l * f.ls + pad(i)] : make_float2(0.f, 0.f); },
-                   [&](int l, int i, float2 v) { dst[l * f.ls + pad(i)] = v; });
+    small_pass<-1, ODD>(f, 0, lines, stw,
+                   [&](int l, int i) { return (xper || i < HALF) ? src[l * f.ls + at<ODD>(i)] : make_float2(0.f, 0.f); },
+                   [&](int l, int i, float2 v) { dst[l * f.ls + at<ODD>(i)] = v; });
   }
-  const float2* Z = small_passes<-1>(f, 1, f.np, lines, stw, Y, X);
+  const float2* Z = small_passes<-1, ODD>(f, 1, f.np, lines, stw, Y, X);
   __syncthreads();
   // 6. Z -> X pairwise and store the half spectrum
   const int items = lines * (HALF + 1);
@@ -435,11 +439,11 @@ __global__ void __launch_bounds__(384, 2) small_row_kernel(const __grid_constant
     const float2 wp = shw[k], wm = cconj(wp);
     float2 xk, xl;
     if (k == 0) {
-      const float2 A = Lz[pad(0)];
+      const float2 A = Lz[at<ODD>(0)];
       xk = make_float2(A.x + A.y, 0.f);
       xl = make_float2(A.x - A.y, 0.f);
     } else {
-      const float2 A = Lz[pad(k)], B = Lz[pad(L - k)];
+      const float2 A = Lz[at<ODD>(k)], B = Lz[at<ODD>(L - k)];
       xk = cscale(csub(cadd(A, cconj(B)), cmul_i<1>(cmul(wp, csub(A, cconj(B))))), 0.5f);
       xl = cscale(cadd(cadd(B, cconj(A)), cmul_i<1>(cmul(wm, csub(B, cconj(A))))), 0.5f);
     }
@@ -504,9 +508,9 @@ __device__ __forceinline__ void z_in_registers(float2 (&x)[3][PZ / 2], KF kfetch
 }
 
 // The z transforms of 16 points take 128 registers or more: TWO runs them at two blocks of 256 threads
-// per SM, otherwise at one of 384.
+// per SM, otherwise at one of 384. ODD: Py is 3 * 2^k or 5 * 2^k.
 __host__ __device__ constexpr int small_conv_threads(int PZ, bool two) { return PZ >= 16 && two ? 256 : 384; }
-template <int PZ, bool TWO = true>
+template <int PZ, bool ODD, bool TWO = true>
 __global__ void __launch_bounds__(small_conv_threads(PZ, TWO), TWO ? 2 : 1) small_conv_kernel(const __grid_constant__ SmallConvArgs s, const float2* __restrict__ tw) {
   const ColArgs& a = s.a;
   const FftPlan& f = s.f;
@@ -527,18 +531,18 @@ __global__ void __launch_bounds__(small_conv_threads(PZ, TWO), TWO ? 2 : 1) smal
   auto gT = [&](int l) { return s.T + ((long long)l * a.Hx + kx) * L; };
   auto from_T = [&]() {
     for (int l = 0; l < lines; ++l)
-      for (int i = tid; i < L; i += T) X[l * f.ls + pad(i)] = gT(l)[i];
+      for (int i = tid; i < L; i += T) X[l * f.ls + at<ODD>(i)] = gT(l)[i];
     __syncthreads();
   };
   auto to_T = [&]() {
     for (int l = 0; l < lines; ++l)
-      for (int i = tid; i < L; i += T) gT(l)[i] = X[l * f.ls + pad(i)];
+      for (int i = tid; i < L; i += T) gT(l)[i] = X[l * f.ls + at<ODD>(i)];
   };
   if (s.phases & 1) {
     float2* dst = X;
-    small_pass<-1>(f, 0, lines, stw, [&](int l, int i) { return i < ny ? gS(l)[i] : make_float2(0.f, 0.f); },
-                   [&](int l, int i, float2 v) { dst[l * f.ls + pad(i)] = v; });
-    float2* R = small_passes<-1>(f, 1, f.np, lines, stw, X, Y);
+    small_pass<-1, ODD>(f, 0, lines, stw, [&](int l, int i) { return i < ny ? gS(l)[i] : make_float2(0.f, 0.f); },
+                   [&](int l, int i, float2 v) { dst[l * f.ls + at<ODD>(i)] = v; });
+    float2* R = small_passes<-1, ODD>(f, 1, f.np, lines, stw, X, Y);
     if (R != X) {
       Y = X;
       X = R;
@@ -556,7 +560,7 @@ __global__ void __launch_bounds__(small_conv_threads(PZ, TWO), TWO ? 2 : 1) smal
       const bool up = ky > L / 2;
       const int kyp = up ? L - ky : ky;
       const float sy = up ? -1.f : 1.f;
-      float2* col = X + pad(ky);
+      float2* col = X + at<ODD>(ky);
       if constexpr (PZ == 1) {
         const float4 k4 = __ldg(a.Kf + (long long)kx * KY + kyp);
         const float kxy = sy * k4.w;
@@ -595,10 +599,10 @@ __global__ void __launch_bounds__(small_conv_threads(PZ, TWO), TWO ? 2 : 1) smal
       return;
     }
   }
-  float2* R = small_passes<1>(f, 0, f.np - 1, lines, stw, X, Y);
+  float2* R = small_passes<1, ODD>(f, 0, f.np - 1, lines, stw, X, Y);
   __syncthreads();
   const float2* src = R;
-  small_pass<1>(f, f.np - 1, lines, stw, [&](int l, int i) { return src[l * f.ls + pad(i)]; },
+  small_pass<1, ODD>(f, f.np - 1, lines, stw, [&](int l, int i) { return src[l * f.ls + at<ODD>(i)]; },
                 [&](int l, int i, float2 v) {
                   if (i < ny) gS(l)[i] = v;
                 });
@@ -666,7 +670,7 @@ bool launch_small_row(int Lx, const RowArgs& a, const float2* tw, cudaStream_t s
   }
   const size_t smem = smem_of(s.staged);
   const int blocks = (a.rows + RB - 1) >> s.rb_log;
-  launch_pdl(small_row_kernel, (unsigned)blocks, (unsigned)small_threads(blocks, 3 * RB * (Lx / 2 + 1), 3 * RB * Lx), smem, st, s, tw);
+  launch_pdl(mixed_len(Lx) ? small_row_kernel<true> : small_row_kernel<false>, (unsigned)blocks, (unsigned)small_threads(blocks, 3 * RB * (Lx / 2 + 1), 3 * RB * Lx), smem, st, s, tw);
   return true;
 }
 
@@ -680,8 +684,7 @@ constexpr long long kSmallFilm = 300000;
 bool small_conv_ok(int Hx, int Py, int Pz, int nz, int per) {
   FftPlan f;
   if (!make_fft_plan(Py, f) || (per & 4) || nz > 8 || Pz == 2) return false;
-  if (nz == 1) return 3LL * Hx * Py <= kSmallFilm;
-  return small_conv_smem(f, nz) <= kSmallSmem;
+  return (nz > 1 || 3LL * Hx * Py <= kSmallFilm) && small_conv_smem(f, nz) <= kSmallSmem;
 }
 
 bool launch_small_conv(const ColArgs& a, float2* S, float2* T, int phases, const float2* tw, cudaStream_t st) {
@@ -698,27 +701,34 @@ bool launch_small_conv(const ColArgs& a, float2* S, float2* T, int phases, const
   const bool two = smem <= kSmallSmem / 2 && a.Hx > kTileBlocks;
   const int values = 3 * a.nz * a.Py;
   const unsigned threads = (unsigned)small_threads(a.Hx, std::max(a.Py, values / 8), values, small_conv_threads(a.Pz, two));
+  auto go = [&](auto pz, auto two_per_sm) {
+    constexpr int PZ = decltype(pz)::value;
+    constexpr bool TWO = decltype(two_per_sm)::value;
+    launch_pdl(mixed_len(a.Py) ? small_conv_kernel<PZ, true, TWO> : small_conv_kernel<PZ, false, TWO>, a.Hx, threads, smem, st, s, tw);
+    return true;
+  };
   switch (a.Pz) {
-    case 1: launch_pdl(small_conv_kernel<1>, a.Hx, threads, smem, st, s, tw); return true;
-    case 4: launch_pdl(small_conv_kernel<4>, a.Hx, threads, smem, st, s, tw); return true;
-    case 8: launch_pdl(small_conv_kernel<8>, a.Hx, threads, smem, st, s, tw); return true;
+    case 1: return go(std::integral_constant<int, 1>(), std::true_type());
+    case 4: return go(std::integral_constant<int, 4>(), std::true_type());
+    case 8: return go(std::integral_constant<int, 8>(), std::true_type());
     case 16:
-      if (two)
-        launch_pdl(small_conv_kernel<16, true>, a.Hx, threads, smem, st, s, tw);
-      else
-        launch_pdl(small_conv_kernel<16, false>, a.Hx, threads, smem, st, s, tw);
-      return true;
+      return two ? go(std::integral_constant<int, 16>(), std::true_type()) : go(std::integral_constant<int, 16>(), std::false_type());
     default: return false;
   }
 }
 
+template <bool ODD>
+static void prepare_small_t() {
+  prep(small_row_kernel<ODD>, kSmallSmem);
+  prep(small_conv_kernel<1, ODD>, kSmallSmem);
+  prep(small_conv_kernel<4, ODD>, kSmallSmem);
+  prep(small_conv_kernel<8, ODD>, kSmallSmem);
+  prep(small_conv_kernel<16, ODD, true>, kSmallSmem);
+  prep(small_conv_kernel<16, ODD, false>, kSmallSmem);
+}
 void prepare_small() {
-  prep(small_row_kernel, kSmallSmem);
-  prep(small_conv_kernel<1>, kSmallSmem);
-  prep(small_conv_kernel<4>, kSmallSmem);
-  prep(small_conv_kernel<8>, kSmallSmem);
-  prep(small_conv_kernel<16, true>, kSmallSmem);
-  prep(small_conv_kernel<16, false>, kSmallSmem);
+  prepare_small_t<false>();
+  prepare_small_t<true>();
 }
 
 }  // namespace gbd
