@@ -66,23 +66,43 @@ __device__ __forceinline__ bool mbar_wait(unsigned long long* b, unsigned parity
 // update, per cell, from the demag field hd of the cell.
 // ---------------------------------------------------------------------------------------------
 
+// Every kernel that ends in this epilogue computes the Laplacian and the update here, with each product
+// and sum's rounding fixed (fmaf, and __fmul_rn / __fadd_rn where the compiler could fuse across a call):
+// left to the compiler, a b + c d fuses one way in one kernel and the other way in the next, and results
+// would depend on the kernel that a launch takes.
+
+// The 7-point Laplacian at a cell c with the neighbours l, r along x, yl, yr along y and zl, zr along z.
+__device__ __forceinline__ float laplacian(const RowArgs& a, float c, float l, float r, float yl, float yr, float zl, float zr) {
+  const float dx = __fadd_rn(fmaf(-2.f, c, l), r), dy = __fadd_rn(fmaf(-2.f, c, yl), yr), dz = __fadd_rn(fmaf(-2.f, c, zl), zr);
+  return fmaf(a.cz, dz, fmaf(a.cy, dy, __fmul_rn(a.cx, dx)));
+}
+
+__device__ __forceinline__ void cross(const float* a, const float* b, float* out) {
+  out[0] = fmaf(a[1], b[2], -__fmul_rn(a[2], b[1]));
+  out[1] = fmaf(a[2], b[0], -__fmul_rn(a[0], b[2]));
+  out[2] = fmaf(a[0], b[1], -__fmul_rn(a[1], b[0]));
+}
+
 // res = H_eff (ROW_HEFF) or dm/dt (ROW_RHS); in RK4 stages the k-sum in acc_out and the next
 // stage's m in mn. m0v / accv: the cell's step-start m and k-sum (stages 2-4).
 __device__ __forceinline__ void llg_update(const RowArgs& a, int mode, const float* hd, const float* m,
                                            const float* lap, const float* m0v, const float* accv, float* mn,
                                            float* acc_out, float* res) {
-  float H[3] = {hd[0] + lap[0] + a.hx, hd[1] + lap[1] + a.hy, hd[2] + lap[2] + a.hz};
+  const float hext[3] = {a.hx, a.hy, a.hz};
+  float H[3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) H[c] = __fadd_rn(__fadd_rn(hd[c], lap[c]), hext[c]);
   if (mode == ROW_HEFF) {
 #pragma unroll
     for (int c = 0; c < 3; ++c) res[c] = H[c];
     return;
   }
   // dm/dt = -gamma/(1+alpha^2) [m x H + alpha m x (m x H)]
-  const float mxH[3] = {m[1] * H[2] - m[2] * H[1], m[2] * H[0] - m[0] * H[2], m[0] * H[1] - m[1] * H[0]};
-  const float mmH[3] = {m[1] * mxH[2] - m[2] * mxH[1], m[2] * mxH[0] - m[0] * mxH[2], m[0] * mxH[1] - m[1] * mxH[0]};
-  float f[3];
+  float mxH[3], mmH[3], f[3];
+  cross(m, H, mxH);
+  cross(m, mxH, mmH);
 #pragma unroll
-  for (int c = 0; c < 3; ++c) f[c] = -a.geff * (mxH[c] + a.alpha * mmH[c]);
+  for (int c = 0; c < 3; ++c) f[c] = __fmul_rn(-a.geff, fmaf(a.alpha, mmH[c], mxH[c]));
   if (mode == ROW_RHS) {
 #pragma unroll
     for (int c = 0; c < 3; ++c) res[c] = f[c];
@@ -92,22 +112,22 @@ __device__ __forceinline__ void llg_update(const RowArgs& a, int mode, const flo
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       acc_out[c] = f[c];
-      mn[c] = m[c] + 0.5f * a.dt * f[c];
+      mn[c] = fmaf(0.5f * a.dt, f[c], m[c]);
     }
   } else if (mode == ROW_RK2 || mode == ROW_RK3) {
     const float h = (mode == ROW_RK2) ? 0.5f * a.dt : a.dt;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      acc_out[c] = accv[c] + 2.f * f[c];
-      mn[c] = m0v[c] + h * f[c];
+      acc_out[c] = fmaf(2.f, f[c], accv[c]);
+      mn[c] = fmaf(h, f[c], m0v[c]);
     }
   } else {  // ROW_RK4
     const float h = a.dt * (1.0f / 6.0f);
 #pragma unroll
-    for (int c = 0; c < 3; ++c) mn[c] = m0v[c] + h * (accv[c] + f[c]);
-    const float inv = rsqrtf(mn[0] * mn[0] + mn[1] * mn[1] + mn[2] * mn[2]);
+    for (int c = 0; c < 3; ++c) mn[c] = fmaf(h, __fadd_rn(accv[c], f[c]), m0v[c]);
+    const float inv = rsqrtf(fmaf(mn[2], mn[2], fmaf(mn[1], mn[1], __fmul_rn(mn[0], mn[0]))));
 #pragma unroll
-    for (int c = 0; c < 3; ++c) mn[c] *= inv;
+    for (int c = 0; c < 3; ++c) mn[c] = __fmul_rn(mn[c], inv);
   }
 }
 
@@ -240,8 +260,8 @@ __device__ __forceinline__ bool epilogue_pair(const RowArgs& a, int mode, int z,
     }
     mv[0][c] = cc.x;
     mv[1][c] = cc.y;
-    lap[0][c] = a.cx * (left - 2.f * cc.x + cc.y) + a.cy * (ym.x - 2.f * cc.x + yp.x) + a.cz * (zm.x - 2.f * cc.x + zp.x);
-    lap[1][c] = a.cx * (cc.x - 2.f * cc.y + right) + a.cy * (ym.y - 2.f * cc.y + yp.y) + a.cz * (zm.y - 2.f * cc.y + zp.y);
+    lap[0][c] = laplacian(a, cc.x, left, cc.y, ym.x, yp.x, zm.x, zp.x);
+    lap[1][c] = laplacian(a, cc.y, cc.x, right, ym.y, yp.y, zm.y, zp.y);
   }
   float m0v[2][3] = {}, accv[2][3] = {};
   if (mode == ROW_RKG) {
@@ -330,10 +350,7 @@ __device__ __forceinline__ bool epilogue_cell(const RowArgs& a, int mode, int z,
     const float* __restrict__ p = a.ms + c * N;
     const float mc = p[idx];
     mv[c] = mc;
-    // (minus - 2 centre + plus) per axis, the operand order of epilogue_pair, so that every
-    // epilogue path rounds alike
-    lap[c] = a.cx * (p[ixm] - 2.f * mc + p[ixp]) + a.cy * (p[iym] - 2.f * mc + p[iyp]) +
-             a.cz * (p[izm] - 2.f * mc + p[izp]);
+    lap[c] = laplacian(a, mc, p[ixm], p[ixp], p[iym], p[iyp], p[izm], p[izp]);
   }
   float m0v[3] = {}, accv[3] = {};
   if (mode == ROW_RKG) {
@@ -640,10 +657,8 @@ __global__ void __launch_bounds__(3 * RB_ * LX / GBD_E,
               }
               mv[0][c] = cc.x;
               mv[1][c] = cc.y;
-              lap[0][c] = a.cx * (left - 2.f * cc.x + cc.y) + a.cy * (ym.x - 2.f * cc.x + yp.x) +
-                          a.cz * (zm.x - 2.f * cc.x + zp.x);
-              lap[1][c] = a.cx * (cc.x - 2.f * cc.y + right) + a.cy * (ym.y - 2.f * cc.y + yp.y) +
-                          a.cz * (zm.y - 2.f * cc.y + zp.y);
+              lap[0][c] = laplacian(a, cc.x, left, cc.y, ym.x, yp.x, zm.x, zp.x);
+              lap[1][c] = laplacian(a, cc.y, cc.x, right, ym.y, yp.y, zm.y, zp.y);
             }
 #pragma unroll
             for (int u = 0; u < 2; ++u) llg_update(a, mode, hd[u], mv[u], lap[u], m0v[u], accv[u], mn[u], ao[u], res[u]);

@@ -76,10 +76,8 @@ __device__ __forceinline__ bool epilogue_rows2(const RowArgs& a, int mode, int z
       const float2 cc = r[u + 1], ym = r[u], yp = r[u + 2];
       mv[u][0][c] = cc.x;
       mv[u][1][c] = cc.y;
-      lap[u][0][c] = a.cx * (left[u] - 2.f * cc.x + cc.y) + a.cy * (ym.x - 2.f * cc.x + yp.x) +
-                     a.cz * (zm[u].x - 2.f * cc.x + zp[u].x);
-      lap[u][1][c] = a.cx * (cc.x - 2.f * cc.y + right[u]) + a.cy * (ym.y - 2.f * cc.y + yp.y) +
-                     a.cz * (zm[u].y - 2.f * cc.y + zp[u].y);
+      lap[u][0][c] = laplacian(a, cc.x, left[u], cc.y, ym.x, yp.x, zm[u].x, zp[u].x);
+      lap[u][1][c] = laplacian(a, cc.y, cc.x, right[u], ym.y, yp.y, zm[u].y, zp[u].y);
     }
   }
   const float hs = rkg && a.hdev ? *a.hdev : 1.f;   // step size on the device, or folded into kw

@@ -274,10 +274,8 @@ __global__ void __launch_bounds__(3 * pipe_rb(LX) * LX / GBD_E, pipe_blocks(K))
           }
           mv[0][c] = cc.x;
           mv[1][c] = cc.y;
-          lap[0][c] = a.cx * (left - 2.f * cc.x + cc.y) + a.cy * (ym.x - 2.f * cc.x + yp.x) +
-                      a.cz * (zm.x - 2.f * cc.x + zp.x);
-          lap[1][c] = a.cx * (cc.x - 2.f * cc.y + right) + a.cy * (ym.y - 2.f * cc.y + yp.y) +
-                      a.cz * (zm.y - 2.f * cc.y + zp.y);
+          lap[0][c] = laplacian(a, cc.x, left, cc.y, ym.x, yp.x, zm.x, zp.x);
+          lap[1][c] = laplacian(a, cc.y, cc.x, right, ym.y, yp.y, zm.y, zp.y);
           if (rk_acc) {
             const float2 q0 = *reinterpret_cast<const float2*>(sM0 + (rr * 3 + c) * LX + x0);
             const float2 qa = *reinterpret_cast<const float2*>(sAc + (rr * 3 + c) * LX + x0);
