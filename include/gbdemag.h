@@ -267,8 +267,9 @@ const char* gbd_last_error(void);
  * of two in [64, 2048], open x axis, nx a multiple of 4, ny a multiple of the group's rows, the
  * staged fields 16-byte aligned; otherwise variant 1 runs). A new mesh starts with variant 1. A
  * variant is the largest tile: a launch that it would spread over fewer blocks than the GPU has
- * SMs takes a smaller one. Some passes have one kernel whatever the variant: the x rows of small
- * meshes, of lengths 3 * 2^k and 5 * 2^k and of most 3D meshes, and the convolution along y and z
+ * SMs takes a smaller one; variant 1 of the x rows also stands for a kernel that transforms two
+ * rows at a time, where that is the faster one. Some passes have one kernel whatever the variant:
+ * the x rows of small meshes and of lengths 3 * 2^k and 5 * 2^k, and the convolution along y and z
  * of small films and of up to 8 layers. All variants give identical
  * results -- each line's FFT and each cell's update do not depend on how lines are grouped --
  * and differ only in speed, which depends on the mesh size. gbd_mesh_autotune times the

@@ -124,8 +124,10 @@ static void set_vec8(RowArgs& a) {
 
 static bool transform_only(const RowArgs& a) { return a.mode == ROW_FWD || (a.mode == ROW_H && !a.extrap); }
 
-// Whether an FP32 launch takes the paired kernel (gbd_rowpair.cuh), whatever the tile variant. It needs
-// an open x. Both sides measured (whole demag or RK stage of the mesh, us, row_kernel / paired):
+static bool rk_stage(const RowArgs& a) { return a.mode >= ROW_RK1 && a.mode <= ROW_RK4; }
+
+// Whether an FP32 launch takes the paired kernel (gbd_rowpair.cuh) in the place of row_kernel's variant 1.
+// It needs an open x. Both sides measured (whole demag or RK stage of the mesh, us, row_kernel / paired):
 //   - lengths 3 * 2^k, 5 * 2^k: always (320x320x4 72 / 61, 1200x600x1 demag 76 / 64; 384x384x64 forward
 //     rows 261 / 132);
 //   - L >= 1024 (one pair per block: half sectors of the spectrum): only stages that row_kernel's staged
@@ -146,18 +148,22 @@ static bool take_pair(int Lx, const RowArgs& a) {
 
 // Tile variants 2 and 3 are the persistent pipelined kernel (gbd_rowpipe.cuh, FP32 only) where it
 // applies (3: the RK stages stage only the spectrum tile, two blocks per SM); other launches of
-// variants 2 and 3 take row_kernel's variant 1.
+// variants 2 and 3 run as variant 1. The variants stay row_kernel's and the pipelined kernel's where they
+// have launches of their own, so that the autotuner can choose them: an RK stage of 256x1024x1
+// takes 26.0 us paired and 22.9 pipelined, of 512x512x1 27.2 and 22.6. H_eff, dm/dt and general RK stages
+// have one kernel, whatever the variant.
 bool launch_row(int Lx, int var, int prec, const RowArgs& a0, const float2* tw, cudaStream_t st) {
   RowArgs a = a0;
   set_vec8(a);
   prec = stage_prec(prec, Lx, false);
   if (prec == 0 && small_row_ok(Lx, a.rows)) return launch_small_row(Lx, a, tw, st);
-  if (prec == 0 && take_pair(Lx, a))
-    return transform_only(a) ? pair_dispatch_io(Lx, &a, tw, st) : pair_dispatch_epi(Lx, &a, tw, st);
-  if (var >= 2 && prec == 0) {
+  if (var >= 2 && prec == 0 && !mixed_len(Lx)) {
     const int kind = pipe_kind(Lx, a, var);
     if (kind >= 0) return pipe_dispatch(Lx, kind, &a, tw, st);
   }
+  const bool has_variants = (rk_stage(a) || transform_only(a)) && !mixed_len(Lx);
+  if (prec == 0 && !(var == 0 && has_variants) && take_pair(Lx, a))
+    return transform_only(a) ? pair_dispatch_io(Lx, &a, tw, st) : pair_dispatch_epi(Lx, &a, tw, st);
   return row_dispatch(Lx, var >= 2 ? 1 : var, prec, &a, tw, st);
 }
 

@@ -1,4 +1,6 @@
-"""The bits of a result do not depend on a field's alignment, which chooses between a kernel's epilogues."""
+"""Tile variants on meshes whose launches depend on them: every row, y and z variant runs the kernel it
+stands for (named by the profiler's trace) and all give the same bits, in one call and split over calls;
+and a field's alignment, which chooses between a kernel's epilogues, does not change its bits either."""
 import numpy as np
 import pytest
 
@@ -8,11 +10,31 @@ from tests.gpu_util import lib, to_dev, to_host
 pytestmark = pytest.mark.gpu
 
 CELL, MS, DT = (3e-9, 3e-9, 3e-9), 8e5, 5e-14
+DEFAULT = (1, 0, 0, 0)
 
 
 @pytest.fixture(scope="module")
 def g():
     return lib()
+
+
+def kernels(call):
+    """Names of the library's kernels that call() launches. (A process's first trace may come back empty.)"""
+    import torch
+    from torch.profiler import ProfilerActivity, profile
+    for _ in range(3):
+        torch.cuda.synchronize()
+        with profile(activities=[ProfilerActivity.CUDA]) as trace:
+            call()
+            torch.cuda.synchronize()
+        names = {e.name.replace("void ", "") for e in trace.events() if "gbd::" in e.name}
+        if names:
+            break
+    return names
+
+
+def has(names, part):
+    return any(part in n for n in names)
 
 
 def run(mesh, m, shift=0):
@@ -35,6 +57,21 @@ def run(mesh, m, shift=0):
     return out
 
 
+@pytest.mark.parametrize("n", [(256, 256, 1), (512, 512, 1), (256, 1024, 1), (1024, 512, 1), (128, 128, 16)])
+def test_row_variants(g, n):
+    m = W.random_unit(n, 51)
+    mesh = g.Mesh(n, CELL, MS, A_ex=1.3e-11, alpha=0.05)
+    base = run(mesh, m)
+    md = to_dev(m)
+    for v in (0, 2, 3):
+        g.gbd_mesh_set_tuning(mesh.handle, (v,) + DEFAULT[1:])
+        for a, b in zip(base, run(mesh, m)):
+            assert np.array_equal(a, b)
+        names = kernels(lambda: mesh.llg_step(md, 1, DT))
+        assert has(names, "row_kernel" if v == 0 else "row_pipe_kernel") and not has(names, "row_pair") and not has(names, "small_row")
+    mesh.close()
+
+
 @pytest.mark.parametrize("n", [(64, 48, 2), (256, 256, 1), (64, 64, 16), (250, 62, 4), (1024, 64, 1), (640, 128, 4), (1000, 60, 1)])
 def test_alignment(g, n):
     m = W.random_unit(n, 53)
@@ -43,4 +80,20 @@ def test_alignment(g, n):
     for shift in (1, 2):
         for a, b in zip(base, run(mesh, m, shift)):
             assert np.array_equal(a, b)
+    mesh.close()
+
+
+def test_y_and_z_variants(g):
+    n = (128, 128, 16)
+    m = W.random_unit(n, 52)
+    mesh = g.Mesh(n, CELL, MS, A_ex=1.3e-11, alpha=0.05)
+    base, ran = run(mesh, m), []
+    H = to_dev(m)
+    for v in ((1, 0, 0, 0), (1, 0, 1, 1)):
+        g.gbd_mesh_set_tuning(mesh.handle, v)
+        for a, b in zip(base, run(mesh, m)):
+            assert np.array_equal(a, b)
+        names = kernels(lambda: mesh.demag(to_dev(m), H))
+        ran.append({n for n in names if "y_pass" in n or "z_conv" in n})
+    assert len(ran[0]) == len(ran[1]) == 3 and not ran[0] & ran[1]
     mesh.close()
