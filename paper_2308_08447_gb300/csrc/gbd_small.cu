@@ -677,13 +677,15 @@ bool launch_small_row(int Lx, const RowArgs& a, const float2* tw, cudaStream_t s
 static size_t small_conv_smem(const FftPlan& f, int nz) { return (size_t)(2 * 3 * nz * f.ls + f.ntw) * sizeof(float2); }
 
 // In one launch: 3D meshes of up to 8 layers whose lines of one kx fit a block's shared memory
-// (RK stage against three launches, us: 32x32x8 26.6 -> 18.5, 480x240x2 45 -> 39, 512x512x4 138 ->
-// 128, 1024x512x2 equal), films up to kSmallFilm values (96x64x1: 13.5 -> 12.9; 200x150x1 17.1 -> 16.0;
-// 256x256x1 equal; 512x512x1 31.8 -> 39.4: film_conv_kernel).
+// (demag against three launches, us: 32x64x4 21 -> 14.5, 480x240x2 42 -> 34, 320x320x4 70 -> 59), films up
+// to kSmallFilm values (96x64x1 stage 13.5 -> 12.9; 200x150x1 17.1 -> 16.0; 256x256x1 equal). Only for
+// lines below 1024 values: one block takes all lines of a kx, and with longer lines its passes and their
+// barriers outlast the launches that it saves (100x512x1 demag 15.6 us by film_conv_kernel, 18.9 here;
+// 512x400x2 47.8 in three launches, 58.6 here; 32x400x4 21.3, 31.0).
 constexpr long long kSmallFilm = 300000;
 bool small_conv_ok(int Hx, int Py, int Pz, int nz, int per) {
   FftPlan f;
-  if (!make_fft_plan(Py, f) || (per & 4) || nz > 8 || Pz == 2) return false;
+  if (Py >= 1024 || !make_fft_plan(Py, f) || (per & 4) || nz > 8 || Pz == 2) return false;
   return (nz > 1 || 3LL * Hx * Py <= kSmallFilm) && small_conv_smem(f, nz) <= kSmallSmem;
 }
 

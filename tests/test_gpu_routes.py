@@ -1,0 +1,36 @@
+"""Which kernel a launch takes at the lines that the dispatch draws (named by the profiler's trace); the
+reasons stand beside the rules. Correctness on both sides of a line is tested elsewhere."""
+import numpy as np
+import pytest
+
+from paper_2308_08447_gb300 import workloads as W
+from tests.gpu_util import lib, to_dev
+from tests.test_gpu_variants import has, kernels
+
+pytestmark = pytest.mark.gpu
+
+CELL, MS = (3e-9, 3e-9, 3e-9), 8e5
+
+
+@pytest.fixture(scope="module")
+def g():
+    return lib()
+
+
+def launched(g, n, what):
+    mesh = g.Mesh(n, CELL, MS, A_ex=1.3e-11, alpha=0.05)
+    m = to_dev(W.random_unit(n, 3))
+    H = to_dev(np.zeros(m.shape))
+    names = kernels({"demag": lambda: mesh.demag(m, H), "heff": lambda: mesh.effective_field(m, H),
+                     "rk4": lambda: mesh.llg_step(m, 1, 1e-14)}[what])
+    mesh.close()
+    return names
+
+
+# the convolution: lines below 1024 values in one launch, longer ones by the tiled kernels
+@pytest.mark.parametrize("n,one", [((100, 256, 1), True), ((100, 257, 1), True), ((100, 512, 1), False), ((20, 1024, 1), False),
+                                   ((300, 320, 2), True), ((512, 400, 2), False)])
+def test_convolution(g, n, one):
+    names = launched(g, n, "demag")
+    assert has(names, "small_conv") == one
+    assert has(names, "film_conv" if n[2] == 1 else "z_conv") == (not one)
