@@ -95,12 +95,17 @@ __host__ __device__ constexpr int zconv_cols_small(int Pz, int prec, int i) {
 // 480x240x2 45.2 / 39.2 / 39.2, 192x224x8 56.7 / 50.7 / 59.9, 512x256x8 114.9 / 108.3 / 116.3.
 constexpr int kTileBlocks = 152;
 // The tile of a launch over `lines` rows, columns or lines: the variant's tile v, or the largest of
-// the smaller ones s0 > s1 > ... (0: none) that spreads the launch over kTileBlocks blocks.
-inline int pick_tile(long long lines, int v, int s0, int s1, int s2 = 0, int s3 = 0) {
+// the smaller ones s0 > s1 > ... (0: none) that spreads the launch over kTileBlocks blocks (or as many as
+// blocks_for asks of the tile before).
+template <class F>
+inline int pick_tile(long long lines, int v, int s0, int s1, int s2, int s3, F blocks_for) {
   int t = v;
   for (int s : {s0, s1, s2, s3})
-    if (s > 0 && s < t && (lines + t - 1) / t < kTileBlocks) t = s;
+    if (s > 0 && s < t && (lines + t - 1) / t < blocks_for(t)) t = s;
   return t;
+}
+inline int pick_tile(long long lines, int v, int s0, int s1, int s2 = 0, int s3 = 0) {
+  return pick_tile(lines, v, s0, s1, s2, s3, [](int) { return kTileBlocks; });
 }
 
 struct RowArgs {

@@ -127,23 +127,31 @@ static bool transform_only(const RowArgs& a) { return a.mode == ROW_FWD || (a.mo
 static bool rk_stage(const RowArgs& a) { return a.mode >= ROW_RK1 && a.mode <= ROW_RK4; }
 
 // Whether an FP32 launch takes the paired kernel (gbd_rowpair.cuh) in the place of row_kernel's variant 1.
-// It needs an open x. Both sides measured (whole demag or RK stage of the mesh, us, row_kernel / paired):
-//   - lengths 3 * 2^k, 5 * 2^k: always (320x320x4 72 / 61, 1200x600x1 demag 76 / 64; 384x384x64 forward
-//     rows 261 / 132);
-//   - L >= 1024 (one pair per block: half sectors of the spectrum): only stages that row_kernel's staged
-//     instances do not serve (800x800x1 63 / 57; with them 1024x1024x1 61.5 / 67, 1024x512x2 106 / 114);
-//   - below, transforms: 3D meshes and films of 1024 rows (256x256x8 58 / 54, 512x512x64 forward rows 204
-//     / 193, 512x1024x1 43 / 39; shorter films 512x512x1 21 / 23);
-//   - below, epilogues: 3D meshes and films that give 90 blocks (480x240x2 39 / 34, 512x512x1 30 / 27,
-//     400x400x1 30 / 26; 256x512x1 15 / 17).
+// It needs an open x. Both sides measured, us, row_kernel / paired:
+//   - lengths 3 * 2^k, 5 * 2^k: always (320x320x4 RK stage 72 / 61, 1200x600x1 demag 76 / 64; 384x384x64
+//     forward rows 261 / 132);
+//   - L >= 1024 (one pair per block: half sectors of the spectrum): of the epilogues those that no staged
+//     instance of row_kernel serves in its RK stages (800x800x1 RK stage 64 / 58, RKF5(6) step 648 / 595;
+//     with staged stages 1024x1024x1 62 / 67, 1024x512x2 106 / 114), and up to L = 2048: at 4096 the paired
+//     epilogues spill (4000x100x1 RK stage 44 / 76, 4000x256x1 equal);
+//   - below, transforms: by the number of row_kernel's tiles of 4096 values. Up to one block per SM it wins
+//     (512x1024x1 demag 30.2 / 37.9, 256x1024x1 18.6 / 26.5, 512x256x4 32.2 / 40.2, 256x512x4 29.5 / 37.4),
+//     unless they are few and 3D (128x64x8 21.2 / 18.8); with a second wave less than half full it loses
+//     (512x1500x1 65 / 56.5), else equal or better on films (512x2000x1 67.9 / 72.3) and worse in 3D
+//     (256x100x32 83 / 73, 512x512x64 forward rows 204 / 193);
+//   - below, epilogues: 3D meshes and films that give 100 blocks (480x240x2 39 / 34, 512x512x1 30 / 27,
+//     400x400x1 27.6 / 26; 128x1500x1, 94 blocks, 27 / 32; 256x512x1 15 / 17).
 // The rule may differ by mode where L is a power of two only: there both kernels round alike, so that a
 // run split over calls, whose first forward rows are a launch of their own, equals the unsplit run.
 static bool take_pair(int Lx, const RowArgs& a) {
   if (mixed_len(Lx)) return true;
-  if ((a.per & 1) || Lx < 32) return false;
+  if ((a.per & 1) || Lx < 32 || Lx > 2048) return false;
   if (Lx >= 1024) return !transform_only(a) && (a.nx % 64 != 0 || a.ny % 4 != 0);
-  if (transform_only(a)) return a.nz > 1 || a.rows >= 1024;
-  return a.nz > 1 || a.rows >= 90 * 2 * (1024 / Lx);
+  if (transform_only(a)) {
+    const long long tiles = ((long long)a.rows * Lx + 4095) / 4096, sms = kTileBlocks;
+    return a.nz > 1 ? tiles < 64 || tiles > sms : tiles > sms && tiles <= sms + sms / 2;
+  }
+  return a.nz > 1 || a.rows >= 100 * 2 * (1024 / Lx);
 }
 
 // Tile variants 2 and 3 are the persistent pipelined kernel (gbd_rowpipe.cuh, FP32 only) where it

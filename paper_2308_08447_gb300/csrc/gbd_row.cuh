@@ -906,11 +906,20 @@ static void row_tiles(F f) {
   if constexpr (S2 > 0) f(std::integral_constant<int, S2>());
 }
 // Launches (a == nullptr: prepares every tile) length LX with the tile of variant var for a's rows.
+// The RK stages ask for a block per SM. Transforms, H_eff and dm/dt, whose smaller blocks read half sectors
+// for less work, ask for 100 blocks, and the latter two up to L = 256 leave eight rows for two only below 64
+// (us, at 152 / as now: 512x1024x1 demag 36.4 / 30.2; 256x2000x1 37.2 / 33.6; 128x1024x1 20.3 / 16.0;
+// 128x512x1 H_eff 26.5 / 16.4. Fewer: 512x400x1 demag with 50 blocks 24.6 against 20.3, 128x1500x1 with 94
+// 27.3 against 22.6).
 template <int LX, int PREC>
 static void row_launch_tile(int var, const RowArgs* a, const float2* tw, cudaStream_t st) {
+  auto blocks_for = [&](int t) {
+    if (a->mode >= ROW_RK1 || a->extrap) return kTileBlocks;
+    return (a->mode == ROW_HEFF || a->mode == ROW_RHS) && LX <= 256 && t <= 8 ? 64 : 100;
+  };
   // (L >= 1024 keeps its four rows: with two, half sectors, 1024x512x1 demag takes 41 us instead of 30)
   const int rb = a ? pick_tile(a->rows, row_rb(LX, var), LX < 1024 ? row_rb(LX, 0) : 0, row_rb_small(LX, PREC, 2),
-                               row_rb_small(LX, PREC, 1), row_rb_small(LX, PREC, 0))
+                               row_rb_small(LX, PREC, 1), row_rb_small(LX, PREC, 0), blocks_for)
                    : 0;
   row_tiles<LX, PREC>([&](auto r) {
     constexpr int RB = decltype(r)::value;

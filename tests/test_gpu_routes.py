@@ -34,3 +34,18 @@ def test_convolution(g, n, one):
     names = launched(g, n, "demag")
     assert has(names, "small_conv") == one
     assert has(names, "film_conv" if n[2] == 1 else "z_conv") == (not one)
+
+
+# x rows of power-of-two lengths: row_kernel's tiles of 4096 values up to one block per SM, the paired rows
+# where they are few (3D) or make a second wave that is less than half full; no paired epilogue at L = 4096
+@pytest.mark.parametrize("n,what,kernel", [((512, 1024, 1), "demag", "row_kernel<512, 8,"), ((128, 1024, 1), "demag", "row_kernel<128, 8,"), ((128, 512, 1), "heff", "row_kernel<128, 8,"),
+                                           ((256, 608, 4), "demag", "row_kernel<256, 16,"), ((256, 152, 4), "demag", "row_pair_kernel<256,"),
+                                           ((512, 1220, 1), "demag", "row_pair_kernel<512,"), ((512, 1830, 1), "demag", "row_kernel<512, 8,"),
+                                           ((512, 399, 1), "rk4", "row_kernel<512,"), ((512, 400, 1), "rk4", "row_pair_kernel<512,"),
+                                           ((2000, 61, 1), "heff", "row_pair_kernel<2048,"), ((4000, 61, 1), "heff", "row_kernel<4096,"),
+                                           ((4000, 61, 1), "rk4", "row_kernel<4096,")])
+def test_power_of_two_rows(g, n, what, kernel):
+    names = launched(g, n, what)
+    assert has(names, kernel), names
+    if what == "demag":
+        assert not has(names, "row_pair" if kernel.startswith("row_kernel") else "row_kernel"), names
