@@ -19,7 +19,8 @@ LIB = os.path.join(HERE, "libgbdemag.so")
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 CUDA_UNITS = ["gbd_api.cu", "gbd_row.cu", "gbd_row_io.cu", "gbd_row_rk.cu", "gbd_row_bf16.cu", "gbd_row_fp16.cu",
-              "gbd_conv.cu", "gbd_conv_bf16.cu", "gbd_conv_fp16.cu", "gbd_ypass.cu", "gbd_mixed_conv.cu", "gbd_small.cu",
+              "gbd_conv.cu", "gbd_conv_bf16.cu", "gbd_conv_fp16.cu", "gbd_ypass.cu", "gbd_mixed_row.cu", "gbd_mixed_conv.cu",
+              "gbd_small.cu",
               "gbd_rowpair.cu", "gbd_rowpair_mixed.cu", "gbd_rowpair_other.cu", "gbd_rowpair_io.cu"]
 CXX_UNITS = ["gbd_tensor.cpp"]
 

@@ -237,8 +237,10 @@ bool pair_dispatch_rk_mixed(int Lx, const RowArgs* a, const float2* tw, cudaStre
 bool pair_dispatch_other(int Lx, const RowArgs* a, const float2* tw, cudaStream_t st);
 bool pair_dispatch_io(int Lx, const RowArgs* a, const float2* tw, cudaStream_t st);
 
-// Transform lengths 3 * 2^k and 5 * 2^k (FP32 only; gbd_mixed_conv.cu): the launchers above forward
-// them here. a == nullptr prepares without launching. False for a length without an instantiation.
+// Transform lengths 3 * 2^k and 5 * 2^k (FP32 only; gbd_mixed_row.cu, gbd_mixed_conv.cu): the launchers
+// above forward them here. a == nullptr prepares without launching. False for a length without an
+// instantiation.
+bool row_dispatch_mixed(int Lx, const RowArgs* a, const float2* tw, cudaStream_t st);
 bool film_dispatch_mixed(int Py, const ColArgs* a, const float2* tw, cudaStream_t st);
 bool ypass_dispatch_mixed(int Py, bool inv, const ColArgs* a, const float2* tw, cudaStream_t st);
 

@@ -128,8 +128,13 @@ static bool rk_stage(const RowArgs& a) { return a.mode >= ROW_RK1 && a.mode <= R
 
 // Whether an FP32 launch takes the paired kernel (gbd_rowpair.cuh) in the place of row_kernel's variant 1.
 // It needs an open x. Both sides measured, us, row_kernel / paired:
-//   - lengths 3 * 2^k, 5 * 2^k: always (320x320x4 RK stage 72 / 61, 1200x600x1 demag 76 / 64; 384x384x64
-//     forward rows 261 / 132);
+//   - lengths 3 * 2^k, 5 * 2^k: where row_kernel's blocks (2048 values over the next power of two) need more
+//     than one wave, the paired rows (320x320x4 RK stage 72 / 61, 1200x600x1 demag 76 / 64, 2500x256x1 66 /
+//     46; 384x384x64 forward rows 261 / 132), and where they leave half of the SMs idle; between, the
+//     transforms run by row_kernel (1500x256x1 demag 34 / 44.6, 700x400x1 29.6 / 36.6, 600x512x1 28.5 /
+//     33.7), and so do the epilogues of 5 * 2^k (RK stage 600x512x1 28.7 / 34.5, 300x1024x1 30.6 / 34.9;
+//     700x512x1 30.2 / 29.1, 1500x256x1 34.3 / 33.3). From L = 2560, where the paired rows spill or leave a
+//     single block per SM, one wave is enough (2500x64x1 demag 31.8 / 36.5, 3000x100x1 RK stage 37.5 / 48.3);
 //   - L >= 1024 (one pair per block: half sectors of the spectrum): of the epilogues those that no staged
 //     instance of row_kernel serves in its RK stages (800x800x1 RK stage 64 / 58, RKF5(6) step 648 / 595;
 //     with staged stages 1024x1024x1 62 / 67, 1024x512x2 106 / 114), and up to L = 2048: at 4096 the paired
@@ -141,10 +146,15 @@ static bool rk_stage(const RowArgs& a) { return a.mode >= ROW_RK1 && a.mode <= R
 //     (256x100x32 83 / 73, 512x512x64 forward rows 204 / 193);
 //   - below, epilogues: 3D meshes and films that give 100 blocks (480x240x2 39 / 34, 512x512x1 30 / 27,
 //     400x400x1 27.6 / 26; 128x1500x1, 94 blocks, 27 / 32; 256x512x1 15 / 17).
-// The rule may differ by mode where L is a power of two only: there both kernels round alike, so that a
-// run split over calls, whose first forward rows are a launch of their own, equals the unsplit run.
+// The rule may differ by mode: both kernels round alike, so that a run split over calls, whose first
+// forward rows are a launch of their own, equals the unsplit run.
 static bool take_pair(int Lx, const RowArgs& a) {
-  if (mixed_len(Lx)) return true;
+  if (mixed_len(Lx)) {
+    const int tiles = (a.rows + row_rb(Lx, 0) - 1) / row_rb(Lx, 0);
+    if (Lx < 320 || tiles > kTileBlocks) return true;
+    if (Lx >= 2560) return false;
+    return tiles < 70 || !(transform_only(a) || odd_part(Lx) == 5);
+  }
   if ((a.per & 1) || Lx < 32 || Lx > 2048) return false;
   if (Lx >= 1024) return !transform_only(a) && (a.nx % 64 != 0 || a.ny % 4 != 0);
   if (transform_only(a)) {
@@ -172,6 +182,7 @@ bool launch_row(int Lx, int var, int prec, const RowArgs& a0, const float2* tw, 
   const bool has_variants = (rk_stage(a) || transform_only(a)) && !mixed_len(Lx);
   if (prec == 0 && !(var == 0 && has_variants) && take_pair(Lx, a))
     return transform_only(a) ? pair_dispatch_io(Lx, &a, tw, st) : pair_dispatch_epi(Lx, &a, tw, st);
+  if (mixed_len(Lx)) return prec == 0 && row_dispatch_mixed(Lx, &a, tw, st);
   return row_dispatch(Lx, var >= 2 ? 1 : var, prec, &a, tw, st);
 }
 
@@ -258,7 +269,10 @@ bool prepare_row(int Lx, int prec) {
     pair_dispatch_io(Lx, nullptr, nullptr, nullptr);
     pair_dispatch_epi(Lx, nullptr, nullptr, nullptr);
   }
-  if (mixed_len(Lx)) return prec <= 0 && pair_dispatch_epi(Lx, nullptr, nullptr, nullptr);
+  if (mixed_len(Lx)) {
+    row_dispatch_mixed(Lx, nullptr, nullptr, nullptr);
+    return prec <= 0 && pair_dispatch_epi(Lx, nullptr, nullptr, nullptr);
+  }
   if (prec <= 0) pipe_dispatch(Lx, -1, nullptr, nullptr, nullptr);
   return row_dispatch(Lx, -1, prec, nullptr, nullptr, nullptr);
 }

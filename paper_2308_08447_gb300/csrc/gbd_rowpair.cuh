@@ -7,8 +7,8 @@
 // value, at the same FMA-pipe time. A block takes NPR row pairs (three pair lines each) and
 // 3 NPR L / 16 threads of 16 pair values. Rows are paired along the flattened (z, y) index; a pair's
 // spectrum is one 16-byte vector of the [kx][y] spectrum where the two rows are adjacent there.
-// For powers of two every operation rounds as row_kernel's, so that a mesh may run its transforms
-// in one kernel and its stages in the other: a run split over calls equals the unsplit run.
+// Every operation rounds as row_kernel's, so that a mesh may run its transforms in one kernel and its
+// stages in the other: a run split over calls equals the unsplit run.
 #pragma once
 #include "gbd_row.cuh"
 

@@ -638,15 +638,17 @@ static bool small_stage_applies(const RowArgs& a, int RB) {
 // kSmallRowMixed): beyond, the fewer instructions per value of row_kernel (row_pair_kernel) win over
 // the shorter chain. RK stage of the whole mesh, us, row_kernel / this kernel: 64x64x1 13.7 / 10.9,
 // 32x32x8 18.5 / 12.5, 128x128x1 14.5 / 11.8, 256x256x1 15.0 / 19.0; mixed lengths, row_pair_kernel /
-// this kernel: 150x150x6 41.8 / 32.4, 600x333x1 demag 44.9 / 39.5, 320x320x4 62.4 / 72.3.
+// this kernel: 150x150x6 41.8 / 32.4, 600x333x1 demag 44.9 / 38.8, 320x320x4 62.4 / 72.3. From L = 768, where
+// two rows fill half of an SM's shared memory, up to 200,000 values (row_kernel / this kernel: 700x320x1
+// demag 33.9 / 38.5, 1200x200x1 30.3 / 32.6, 700x256x1 27.8 / 26.0).
 // One row per block up to 64 rows or kSmallRowOne values, else two (a 16-byte piece of the spectrum):
 // 128x128x1 11.8 / 12.5 us, 256x128x1 15.0 / 13.4, 200x150x1 18.9 / 14.3.
-constexpr long long kSmallRowWork = 40960, kSmallRowMixed = 262144, kSmallRowOne = 20480;
+constexpr long long kSmallRowWork = 40960, kSmallRowMixed = 262144, kSmallRowMixed2 = 200000, kSmallRowOne = 20480;
 
 bool small_row_ok(int Lx, int rows) {
   FftPlan f;
-  return Lx <= 1280 && rows < 65536 && (long long)rows * Lx <= (mixed_len(Lx) ? kSmallRowMixed : kSmallRowWork) &&
-         make_fft_plan(Lx, f);
+  const long long most = !mixed_len(Lx) ? kSmallRowWork : Lx >= 768 ? kSmallRowMixed2 : kSmallRowMixed;
+  return Lx <= 1280 && rows < 65536 && (long long)rows * Lx <= most && make_fft_plan(Lx, f);
 }
 
 bool launch_small_row(int Lx, const RowArgs& a, const float2* tw, cudaStream_t st) {

@@ -49,3 +49,30 @@ def test_power_of_two_rows(g, n, what, kernel):
     assert has(names, kernel), names
     if what == "demag":
         assert not has(names, "row_pair" if kernel.startswith("row_kernel") else "row_kernel"), names
+
+
+# x rows of lengths 3 * 2^k and 5 * 2^k: row_kernel where its blocks make one wave that fills half of the SMs
+@pytest.mark.parametrize("n,what,kernel", [((700, 300, 1), "demag", "row_kernel<768,"), ((700, 608, 1), "demag", "row_kernel<768,"),
+                                           ((700, 609, 1), "demag", "row_pair_kernel<768,"), ((700, 400, 1), "rk4", "row_pair_kernel<768,"),
+                                           ((600, 512, 1), "rk4", "row_kernel<640,"), ((300, 304, 4), "demag", "row_kernel<320,"),
+                                           ((1500, 138, 1), "demag", "row_pair_kernel<1536,"), ((1500, 140, 1), "demag", "row_kernel<1536,"),
+                                           ((2500, 16, 1), "heff", "row_kernel<2560,"), ((2500, 153, 1), "heff", "row_pair_kernel<2560,"),
+                                           ((3000, 16, 1), "rk4", "row_kernel<3072,"), ((180, 1400, 1), "demag", "row_pair_kernel<192,"),
+                                           ((600, 333, 1), "demag", "small_row_kernel"), ((700, 260, 1), "demag", "small_row_kernel")])
+def test_mixed_rows(g, n, what, kernel):
+    assert has(launched(g, n, what), kernel)
+
+
+@pytest.mark.parametrize("n", [(700, 400, 1), (1500, 256, 1), (640, 103, 6), (128, 1024, 1), (250, 160, 8)])
+def test_kernels_of_a_run_round_alike(g, n):
+    # the first forward transform and the stages run in different kernels: a split run equals the unsplit one
+    import torch
+    m = to_dev(W.vortex_noise(n, CELL, 12))
+    mesh = g.Mesh(n, CELL, MS, A_ex=1.3e-11, alpha=0.05)
+    one, split = m.clone(), m.clone()
+    mesh.llg_step(one, 4, 5e-14)
+    for k in (1, 2, 1):
+        mesh.llg_step(split, k, 5e-14)
+    torch.cuda.synchronize()
+    assert torch.equal(one, split)
+    mesh.close()
