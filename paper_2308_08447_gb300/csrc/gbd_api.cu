@@ -1477,7 +1477,7 @@ extern "C" gbd_status gbd_demag_noalloc(gbd_mesh* m, const float* M, float* H, v
 // Each kernel family has two tile shapes (lines per block; gbd_kernels.cuh). They compute the
 // same numbers -- every line's transform and every cell's update is independent of how lines
 // are grouped into blocks -- so the choice only changes speed. gbd_mesh_autotune times both
-// shapes of each pass the mesh uses, on the mesh's own (zeroed) buffers, keeps the faster one,
+// shapes of each pass whose launches on this mesh have them, on the mesh's own (zeroed) buffers, keeps the faster one,
 // and caches the choice by mesh size and device: in the process, and in the text file named
 // by GBD_AUTOTUNE_CACHE when that is set (lines "gbd<generation> nx ny nz device Px Py precision var_row
 // var_film var_y var_z pow2 var_row_io"). A choice holds for the kernels it was timed on: lines of
@@ -1593,7 +1593,9 @@ bool can_pad_pow2(const gbd_mesh* m) {
 // mesh's own buffers (zeroed by the caller).
 cudaError_t time_demag_passes(gbd_mesh* m, cudaStream_t st, float* ms) {
   gbd::RowArgs a = row_args(m);
-  return time_variant(st, 5, [&] {
+  const int tracing = m->timing;
+  m->timing = 0;   // traced launches would be counted, and the convolution split into its passes
+  const cudaError_t e = time_variant(st, 5, [&] {
     a.in = m->bufA;
     a.mode = gbd::ROW_FWD;
     a.fwd_after = 1;
@@ -1604,6 +1606,8 @@ cudaError_t time_demag_passes(gbd_mesh* m, cudaStream_t st, float* ms) {
     a.fwd_after = 0;
     gbd::launch_row(m->p.Lx, row_var(m, a.mode), m->p.prec, a, m->tw, st);
   }, ms);
+  m->timing = tracing;
+  return e;
 }
 
 // A scratch copy of m planned on powers of two (kernel spectrum zero: for timing only), tuned.
@@ -1741,10 +1745,11 @@ extern "C" gbd_status gbd_mesh_autotune(gbd_mesh* m, void* stream) {
   ra.acc = m->acc;
   ra.mode = gbd::ROW_RK2;
   ra.fwd_after = 1;
-  e = pick(0, [&](int v) { gbd::launch_row(p.Lx, v, p.prec, ra, m->tw, st); }, p.prec == 0 ? 4 : 2);
+  const bool rows_vary = gbd::row_has_variants(p.Lx, p.prec, ra.rows);
+  if (rows_vary) e = pick(0, [&](int v) { gbd::launch_row(p.Lx, v, p.prec, ra, m->tw, st); }, p.prec == 0 ? 4 : 2);
   // the transform-only x-row launches: a forward transform and an inverse one to H_d
   int best_io = p.var_row_io;
-  if (e == cudaSuccess) {
+  if (e == cudaSuccess && rows_vary) {
     gbd::RowArgs fa = row_args(m), ia = row_args(m);
     fa.in = m->bufA;
     fa.mode = gbd::ROW_FWD;
@@ -1766,7 +1771,9 @@ extern "C" gbd_status gbd_mesh_autotune(gbd_mesh* m, void* stream) {
     }
   }
   gbd::ColArgs ca = col_args(m);
-  if (e == cudaSuccess && p.film) {
+  if (conv_in_one(p)) {
+    // one kernel, no variants
+  } else if (e == cudaSuccess && p.film) {
     ca.dst = m->S;
     ca.Kf = static_cast<const float4*>(m->K);
     e = pick(1, [&](int v) { gbd::launch_film_conv(v, p.prec, ca, m->tw, st); });

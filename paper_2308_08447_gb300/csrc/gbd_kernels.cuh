@@ -204,6 +204,8 @@ struct ColArgs {
 // prec: 0 FP32 stages; 1 / 2 radix-16 stages on the tensor cores in split BF16 / split FP16
 // (gbd_tc.cuh).
 bool launch_row(int Lx, int var, int prec, const RowArgs& a, const float2* tw, cudaStream_t st);
+// Whether the tile variants of a mesh's x rows differ (else one kernel serves them all).
+bool row_has_variants(int Lx, int prec, int rows);
 // An extrapolated RK4 stage with no forward transform after it (a.extrap = 1, a.fwd_after = 0):
 // the row kernel's epilogue alone, at full occupancy.
 void launch_extrap_stage(const RowArgs& a, cudaStream_t st);

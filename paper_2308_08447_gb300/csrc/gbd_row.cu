@@ -186,6 +186,10 @@ bool launch_row(int Lx, int var, int prec, const RowArgs& a0, const float2* tw, 
   return row_dispatch(Lx, var >= 2 ? 1 : var, prec, &a, tw, st);
 }
 
+bool row_has_variants(int Lx, int prec, int rows) {
+  return stage_prec(prec, Lx, false) != 0 || !(mixed_len(Lx) || small_row_ok(Lx, rows));
+}
+
 // One warp: lane l writes register r of each table at word r * 32 + l (Dft16Frags::load).
 __global__ void __launch_bounds__(32) dft16_frag_kernel(unsigned* frag) {
   const int lane = threadIdx.x & 31;

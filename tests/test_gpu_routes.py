@@ -76,3 +76,19 @@ def test_kernels_of_a_run_round_alike(g, n):
     torch.cuda.synchronize()
     assert torch.equal(one, split)
     mesh.close()
+
+
+# the autotuner times what the mesh runs: nothing for passes with one kernel
+@pytest.mark.parametrize("n,not_timed,timed", [((96, 60, 1), ("film_conv", "row_kernel", "row_pipe"), None),
+                                               ((72, 52, 6), ("y_pass", "z_conv", "row_kernel", "row_pipe"), None),
+                                               ((260, 244, 2), ("y_pass", "z_conv", "film_conv"), "row_pipe"),
+                                               ((256, 268, 1), (), "film_conv")])
+def test_autotuner_times_what_runs(g, n, not_timed, timed):
+    launched(g, n, "demag")               # a process's first trace may be empty, and tuning runs once
+    mesh = g.Mesh(n, CELL, MS, pow2_pad=True)
+    names = kernels(mesh.autotune)
+    assert not any(has(names, part) for part in not_timed)
+    assert timed is None or has(names, timed)
+    if timed is None:
+        assert g.gbd_mesh_get_tuning(mesh.handle) == (1, 0, 0, 0)
+    mesh.close()
