@@ -48,12 +48,12 @@ __host__ __device__ constexpr int row_rb(int Lx, int v) {
 }
 // Smaller row tiles, for meshes whose rows would fill too few of them: the row counts below the
 // variant's that have kernels -- 2 rows (one 16-byte vector of the [kx][y] spectrum) or as many
-// as give a block 48 threads, and four and sixteen times that. The tensor-core passes need whole warps.
+// as give a block 48 threads, and four times that. The tensor-core passes need whole warps.
 __host__ __device__ constexpr int row_rb_min(int Lx, int prec) {
   return prec != 0 ? (Lx >= 256 ? 2 : Lx >= 16 ? 512 / Lx : row_rb(Lx, 0))
                    : (pow2_floor(Lx) >= 128 ? 2 : Lx >= 16 ? 256 / pow2_floor(Lx) : row_rb(Lx, 0));
 }
-__host__ __device__ constexpr int row_rb_small(int Lx, int prec, int i) {   // i = 0, 1, 2 (0: none)
+__host__ __device__ constexpr int row_rb_small(int Lx, int prec, int i) {   // i = 0, 1 (0: none)
   return (row_rb_min(Lx, prec) << (2 * i)) < row_rb(Lx, 0) ? row_rb_min(Lx, prec) << (2 * i) : 0;
 }
 // kx columns per film-convolution block (3 lines each)
@@ -98,14 +98,14 @@ constexpr int kTileBlocks = 152;
 // the smaller ones s0 > s1 > ... (0: none) that spreads the launch over kTileBlocks blocks (or as many as
 // blocks_for asks of the tile before).
 template <class F>
-inline int pick_tile(long long lines, int v, int s0, int s1, int s2, int s3, F blocks_for) {
+inline int pick_tile(long long lines, int v, int s0, int s1, int s2, F blocks_for) {
   int t = v;
-  for (int s : {s0, s1, s2, s3})
+  for (int s : {s0, s1, s2})
     if (s > 0 && s < t && (lines + t - 1) / t < blocks_for(t)) t = s;
   return t;
 }
-inline int pick_tile(long long lines, int v, int s0, int s1, int s2 = 0, int s3 = 0) {
-  return pick_tile(lines, v, s0, s1, s2, s3, [](int) { return kTileBlocks; });
+inline int pick_tile(long long lines, int v, int s0, int s1, int s2) {
+  return pick_tile(lines, v, s0, s1, s2, [](int) { return kTileBlocks; });
 }
 
 struct RowArgs {

@@ -895,15 +895,13 @@ static void row_launch_t(const RowArgs* a, const float2* tw, cudaStream_t st) {
 template <int LX, int PREC, class F>
 static void row_tiles(F f) {
   constexpr int V0 = row_rb(LX, 0), V1 = row_rb(LX, 1);
-  constexpr int S0 = row_rb_small(LX, PREC, 0), S1 = row_rb_small(LX, PREC, 1), S2 = row_rb_small(LX, PREC, 2);
+  constexpr int S0 = row_rb_small(LX, PREC, 0), S1 = row_rb_small(LX, PREC, 1);
   if (f(std::integral_constant<int, V0>())) return;
   if constexpr (V1 != V0)
     if (f(std::integral_constant<int, V1>())) return;
   if constexpr (S0 > 0)
     if (f(std::integral_constant<int, S0>())) return;
-  if constexpr (S1 > 0)
-    if (f(std::integral_constant<int, S1>())) return;
-  if constexpr (S2 > 0) f(std::integral_constant<int, S2>());
+  if constexpr (S1 > 0) f(std::integral_constant<int, S1>());
 }
 // Launches (a == nullptr: prepares every tile) length LX with the tile of variant var for a's rows.
 // The RK stages ask for a block per SM. Transforms, H_eff and dm/dt, whose smaller blocks read half sectors
@@ -918,8 +916,8 @@ static void row_launch_tile(int var, const RowArgs* a, const float2* tw, cudaStr
     return (a->mode == ROW_HEFF || a->mode == ROW_RHS) && LX <= 256 && t <= 8 ? 64 : 100;
   };
   // (L >= 1024 keeps its four rows: with two, half sectors, 1024x512x1 demag takes 41 us instead of 30)
-  const int rb = a ? pick_tile(a->rows, row_rb(LX, var), LX < 1024 ? row_rb(LX, 0) : 0, row_rb_small(LX, PREC, 2),
-                               row_rb_small(LX, PREC, 1), row_rb_small(LX, PREC, 0), blocks_for)
+  const int rb = a ? pick_tile(a->rows, row_rb(LX, var), LX < 1024 ? row_rb(LX, 0) : 0, row_rb_small(LX, PREC, 1),
+                               row_rb_small(LX, PREC, 0), blocks_for)
                    : 0;
   row_tiles<LX, PREC>([&](auto r) {
     constexpr int RB = decltype(r)::value;

@@ -14,7 +14,7 @@
 
 namespace gbd {
 
-// Row pairs per block: 192 threads (more for L above 1024).
+// Row pairs per block: 192 threads (240 and 288 for lengths 5 * 2^k and 3 * 2^k; more for L above 1024).
 __host__ __device__ constexpr int pair_npr(int L) { return 1024 / pow2_floor(L) > 0 ? 1024 / pow2_floor(L) : 1; }
 __host__ __device__ constexpr int pair_threads(int L, int npr) { return 3 * npr * L / GBD_E; }
 // Blocks per SM: the epilogue's instances at 12 to 16 warps (168 or 128 registers; at 96 they spill and
@@ -482,7 +482,6 @@ static bool pair_switch(int L, F f) {
       GBD_PAIR_LEN(512)
       GBD_PAIR_LEN(1024)
       GBD_PAIR_LEN(2048)
-      GBD_PAIR_LEN(4096)
       default: return false;
     }
   } else {

@@ -662,7 +662,7 @@ bool launch_small_row(int Lx, const RowArgs& a, const float2* tw, cudaStream_t s
   s.mnx = magic_div(a.nx);
   s.mpad = magic_div(std::max(1, Lx - a.nx));
   s.mny = magic_div(a.ny);
-  // stage what leaves room for two blocks per SM
+  // stage the input rows where they fit, the others while that leaves room for two blocks per SM
   auto smem_of = [&](int staged) { return small_row_smem(s.f, RB, a.nx, small_stage_rows(RB, staged)); };
   s.staged = 0;
   if (small_stage_applies(a, RB) && smem_of(1) <= kSmallSmem) {
