@@ -1593,9 +1593,7 @@ bool can_pad_pow2(const gbd_mesh* m) {
 // mesh's own buffers (zeroed by the caller).
 cudaError_t time_demag_passes(gbd_mesh* m, cudaStream_t st, float* ms) {
   gbd::RowArgs a = row_args(m);
-  const int tracing = m->timing;
-  m->timing = 0;   // traced launches would be counted, and the convolution split into its passes
-  const cudaError_t e = time_variant(st, 5, [&] {
+  return time_variant(st, 5, [&] {
     a.in = m->bufA;
     a.mode = gbd::ROW_FWD;
     a.fwd_after = 1;
@@ -1606,9 +1604,16 @@ cudaError_t time_demag_passes(gbd_mesh* m, cudaStream_t st, float* ms) {
     a.fwd_after = 0;
     gbd::launch_row(m->p.Lx, row_var(m, a.mode), m->p.prec, a, m->tw, st);
   }, ms);
-  m->timing = tracing;
-  return e;
 }
+
+// No tracing while the autotuner times: traced launches would be counted, and the convolution split
+// into its passes.
+struct Untraced {
+  gbd_mesh* m;
+  int timing;
+  explicit Untraced(gbd_mesh* mesh) : m(mesh), timing(mesh->timing) { m->timing = 0; }
+  ~Untraced() { m->timing = timing; }
+};
 
 // A scratch copy of m planned on powers of two (kernel spectrum zero: for timing only), tuned.
 gbd_status make_pow2_twin(gbd_mesh* m, void* stream, gbd_mesh** out) {
@@ -1711,6 +1716,7 @@ extern "C" gbd_status gbd_mesh_autotune(gbd_mesh* m, void* stream) {
       return GBD_OK;
     }
   }
+  const Untraced untraced(m);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   // zeroed buffers keep every timed pass finite
   cudaError_t e = cudaSuccess;
@@ -1720,7 +1726,7 @@ extern "C" gbd_status gbd_mesh_autotune(gbd_mesh* m, void* stream) {
   if (e == cudaSuccess) e = cudaMemsetAsync(m->bufA, 0, p.bytes_state / 3, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(m->bufB, 0, p.bytes_state / 3, st);
   if (e != cudaSuccess) return cuda_fail(e, "gbd_mesh_autotune: memset");
-  const int reps = 5;
+  const int reps = 20;
   std::array<int, 4> best = {p.var_row, p.var_film, p.var_y, p.var_z};
   auto pick = [&](int slot, auto launch_v, int nvar = 2) -> cudaError_t {
     float t[4];
@@ -1736,7 +1742,9 @@ extern "C" gbd_status gbd_mesh_autotune(gbd_mesh* m, void* stream) {
     best[slot] = b;
     return cudaSuccess;
   };
-  // x rows: an RK4 middle stage with the next forward transform, on zeroed state
+  // x rows: an RK4 middle stage with the next forward transform, on zeroed state, after its convolution
+  // (launched alone, back to back, the rows find their spectrum in other caches and start on empty SMs:
+  // the choice lost up to a quarter of a step)
   gbd::RowArgs ra = row_args(m);
   ra.dt = 1e-13f;
   ra.ms = m->bufA;
@@ -1746,8 +1754,12 @@ extern "C" gbd_status gbd_mesh_autotune(gbd_mesh* m, void* stream) {
   ra.mode = gbd::ROW_RK2;
   ra.fwd_after = 1;
   const bool rows_vary = gbd::row_has_variants(p.Lx, p.prec, ra.rows);
-  if (rows_vary) e = pick(0, [&](int v) { gbd::launch_row(p.Lx, v, p.prec, ra, m->tw, st); }, p.prec == 0 ? 4 : 2);
-  // the transform-only x-row launches: a forward transform and an inverse one to H_d
+  if (rows_vary)
+    e = pick(0, [&](int v) {
+      enqueue_conv(m, m->S, m->T, st);
+      gbd::launch_row(p.Lx, v, p.prec, ra, m->tw, st);
+    }, p.prec == 0 ? 4 : 2);
+  // the transform-only x-row launches, around the convolution: a forward transform and an inverse one to H_d
   int best_io = p.var_row_io;
   if (e == cudaSuccess && rows_vary) {
     gbd::RowArgs fa = row_args(m), ia = row_args(m);
@@ -1761,6 +1773,7 @@ extern "C" gbd_status gbd_mesh_autotune(gbd_mesh* m, void* stream) {
     for (int v = 0; v < nv && e == cudaSuccess; ++v)
       e = time_variant(st, reps, [&] {
         gbd::launch_row(p.Lx, v, p.prec, fa, m->tw, st);
+        enqueue_conv(m, m->S, m->T, st);
         gbd::launch_row(p.Lx, v, p.prec, ia, m->tw, st);
       }, &t[v]);
     if (e == cudaSuccess) {
