@@ -132,7 +132,8 @@ static bool rk_stage(const RowArgs& a) { return a.mode >= ROW_RK1 && a.mode <= R
 //     than one wave, the paired rows (320x320x4 RK stage 72 / 61, 1200x600x1 demag 76 / 64, 2500x256x1 66 /
 //     46; 384x384x64 forward rows 261 / 132), and where they leave half of the SMs idle; between, the
 //     transforms run by row_kernel (1500x256x1 demag 34 / 44.6, 700x400x1 29.6 / 36.6, 600x512x1 28.5 /
-//     33.7), and so do the epilogues of 5 * 2^k (RK stage 600x512x1 28.7 / 34.5, 300x1024x1 30.6 / 34.9;
+//     33.7), and so do the epilogues of 5 * 2^k (RK stage 600x512x1 28.7 / 34.5, 300x1024x1 30.6 / 34.9; but
+//     300x256x4 43.5 / 43.1, and among the meshes of a batch the paired rows leave more of an SM free;
 //     700x512x1 30.2 / 29.1, 1500x256x1 34.3 / 33.3). From L = 2560, where the paired rows spill or leave a
 //     single block per SM, one wave is enough (2500x64x1 demag 31.8 / 36.5, 3000x100x1 RK stage 37.5 / 48.3);
 //   - L >= 1024 (one pair per block: half sectors of the spectrum): of the epilogues those that no staged
@@ -153,7 +154,7 @@ static bool take_pair(int Lx, const RowArgs& a) {
     const int tiles = (a.rows + row_rb(Lx, 0) - 1) / row_rb(Lx, 0);
     if (Lx < 320 || tiles > kTileBlocks) return true;
     if (Lx >= 2560) return false;
-    return tiles < 70 || !(transform_only(a) || odd_part(Lx) == 5);
+    return tiles < 70 || !(transform_only(a) || (odd_part(Lx) == 5 && (a.nz == 1 || Lx >= 640)));
   }
   if ((a.per & 1) || Lx < 32 || Lx > 2048) return false;
   if (Lx >= 1024) return !transform_only(a) && (a.nx % 64 != 0 || a.ny % 4 != 0);

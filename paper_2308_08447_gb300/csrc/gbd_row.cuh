@@ -908,11 +908,11 @@ static void row_tiles(F f) {
 // for less work, ask for 100 blocks, and the latter two up to L = 256 leave eight rows for two only below 64
 // (us, at 152 / as now: 512x1024x1 demag 36.4 / 30.2; 256x2000x1 37.2 / 33.6; 128x1024x1 20.3 / 16.0;
 // 128x512x1 H_eff 26.5 / 16.4. Fewer: 512x400x1 demag with 50 blocks 24.6 against 20.3, 128x1500x1 with 94
-// 27.3 against 22.6).
+// 27.3 against 22.6). The split precisions keep a block per SM throughout (128x128x8 demag 40.2 / 41.5).
 template <int LX, int PREC>
 static void row_launch_tile(int var, const RowArgs* a, const float2* tw, cudaStream_t st) {
   auto blocks_for = [&](int t) {
-    if (a->mode >= ROW_RK1 || a->extrap) return kTileBlocks;
+    if (PREC != 0 || a->mode >= ROW_RK1 || a->extrap) return kTileBlocks;
     return (a->mode == ROW_HEFF || a->mode == ROW_RHS) && LX <= 256 && t <= 8 ? 64 : 100;
   };
   // (L >= 1024 keeps its four rows: with two, half sectors, 1024x512x1 demag takes 41 us instead of 30)
