@@ -91,8 +91,8 @@ __host__ __device__ constexpr int zconv_cols_small(int Pz, int prec, int i) {
 // A launch takes a smaller tile while its own spreads it over fewer blocks than the GPU has SMs. A
 // block takes the same ~10 us on an empty SM whatever its tile, so idle SMs cost in proportion; but
 // twice as many blocks as SMs is already slower where the tile's half sectors and barriers count.
-// RK stage, us, by the number of blocks asked for (none / 152 / 304): 96x64x1 24.3 / 13.5 / 13.5,
-// 480x240x2 45.2 / 39.2 / 39.2, 192x224x8 56.7 / 50.7 / 59.9, 512x256x8 114.9 / 108.3 / 116.3.
+// RK stage, us, by the number of blocks asked for (none / 152 / 304): 192x224x8 56.7 / 50.7 / 59.9,
+// 512x256x8 114.9 / 108.3 / 116.3.
 constexpr int kTileBlocks = 152;
 // The tile of a launch over `lines` rows, columns or lines: the variant's tile v, or the largest of
 // the smaller ones s0 > s1 > ... (0: none) that spreads the launch over kTileBlocks blocks (or as many as

@@ -8,13 +8,13 @@
 namespace gbd {
 
 __host__ __device__ constexpr int min_blocks(int T) { return T >= 768 ? 1 : 768 / T; }
-// The FP32 convolution kernels run at 1152 threads per SM (three blocks of 384 at <= 56
-// registers): the film's fused pass holds at most two components' values at a time, and the
-// 3D z convolution splits its fused pass into per-component butterflies and a product phase.
+// The FP32 film convolution runs at 1152 threads per SM (three blocks of 384 at <= 56 registers): its
+// fused pass holds at most two components' values at a time. (The 3D z convolution holds three and runs at
+// 24 warps, zconv_blocks.)
 __host__ __device__ constexpr int min_blocks_film(int T) { return T >= 1152 ? 1 : 1152 / T; }
 
-// Programmatic dependent launch (PTX griddepcontrol): the x-row kernels, the film convolution and
-// the extrapolated RK stage are launched with programmatic stream serialization, so a launch may
+// Programmatic dependent launch (PTX griddepcontrol): the x-row kernels, the convolution kernels (film, y
+// passes, z, one-launch) and the extrapolated RK stage are launched with programmatic stream serialization, so a launch may
 // begin while the kernel before it in the stream still runs -- its blocks become resident on SMs
 // the predecessor has left idle. Every thread waits for the predecessor grid to complete with its
 // memory operations visible before it touches memory the predecessor may write; the block then

@@ -616,7 +616,7 @@ constexpr size_t kSmallSmem = 232448;   // dynamic shared memory of a block
 constexpr int kSmallThreads = 384;
 
 // Threads of a block: one per x-row item or y frequency while the blocks leave SMs to spare (96x64x1
-// stage 10.4 -> 9.1 us), else one per eight values (the eight-mesh batch 6620 -> 6370 us).
+// stage 10.4 -> 9.1 us), else one per eight values (4 % of the eight-mesh batch).
 static int small_threads(int blocks, int items, int values, int most = kSmallThreads) {
   const int t = blocks <= 2 * kTileBlocks ? items : values / 8;
   return std::min(most, (t + 31) / 32 * 32);
